@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "hubrows.cuh"
 #include "kernels.cuh"
 #include "msbicg_impl.cuh"
 #include "profile.cuh"
@@ -132,6 +133,28 @@ __global__ void __launch_bounds__(256) k_lz_apply(View op, const V* __restrict__
     }
     store_partials<1>(acc, sm, part);
 }
+
+// The same for one real FP64 vector as the epilogue of the row-tiled Hubbard product.
+struct LzEpi {
+    double* w;
+    const double* qp;
+    const double* bprev;
+    double* part;
+    double bp, dot;
+    __device__ __forceinline__ bool stop() const { return false; }
+    __device__ __forceinline__ void begin(int) { bp = bprev[0]; }
+    __device__ __forceinline__ void operator()(int64_t s, double xs, double acc, double dg, double mt) {
+        double h = fma(mt, acc, dg * xs);
+        if (bp != 0.0) h = fma(-bp, qp[s], h);
+        w[s] = h;
+        dot = fma(xs, h, dot);
+    }
+    __device__ __forceinline__ void pair(int64_t, float2, float2, float2, float2, float, float, float) {}
+    __device__ __forceinline__ void finish(double* sm) {
+        double acc[1] = {dot};
+        store_partials<1>(acc, sm, part);
+    }
+};
 
 // a_c = sum of partials (one CTA per active column).
 __global__ void k_lz_sum(const double* part, int nblk, const int* cols, double* out, int64_t stride_k, int k) {
@@ -284,7 +307,8 @@ struct GroundScratch {
     double* bcur;     // 1
     double* n0;       // 1
     int* col0;        // 1
-    double* part;     // 3 * grid
+    double* part;     // part_n partial sums: at least 3 per block, and one per CTA of the
+    int part_n;       // row-tiled product
 };
 
 template <class View>
@@ -292,6 +316,9 @@ static void lanczos_ground(const msb_op* op, const View& view, int64_t n, double
                            double* g, const GroundScratch& S, int grid, GroundResult& out, cudaStream_t st) {
     const double vb = 8.0 * double(n);                       // one real FP64 vector
     const double hxf = 0.5 * op->hx_flops();
+    RowPlan rows;
+    if constexpr (std::is_same<View, HubView>::value) rows = row_plan<double>(op, 1);
+    rows.ok = rows.ok && rows.grid <= S.part_n;
     MSB_CUDA(cudaMemsetAsync(S.col0, 0, sizeof(int), st));
     if (start) MSB_CUDA(cudaMemcpyAsync(S.v0, start, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
     else { k_fill_start<<<grid, 256, 0, st>>>(S.v0, n, 0x5EEDull); ++out.launches; }
@@ -314,9 +341,15 @@ static void lanczos_ground(const msb_op* op, const View& view, int64_t n, double
             if (accumulate && k == kmax - 1) break;
             {
                 ProfScope ps("ground_state", st, 3 * vb + op->matrix_bytes(8), hxf + 4.0 * n);
-                k_lz_apply<View, double><<<dim3(grid, 1), 256, 0, st>>>(view, q, qp, w, n, S.col0, S.bcur, S.part);
+                if (rows.ok)
+                    launch_hub_rows<double>(rows, nullptr, q, n, 1, 0.0, LzEpi{w, qp, S.bcur, S.part, 0.0, 0.0}, st);
+                else
+                    k_lz_apply<View, double><<<dim3(grid, 1), 256, 0, st>>>(view, q, qp, w, n, S.col0, S.bcur, S.part);
             }
-            { ProfScope ps("ground_state", st, 0, 0); k_lz_sum<<<1, 256, 0, st>>>(S.part, grid, S.col0, S.a, 1, k); }
+            {
+                ProfScope ps("ground_state", st, 0, 0);
+                k_lz_sum<<<1, 256, 0, st>>>(S.part, rows.ok ? rows.grid : grid, S.col0, S.a, 1, k);
+            }
             {
                 ProfScope ps("ground_state", st, 3 * vb, 4.0 * n);
                 k_lz_orth<double><<<dim3(grid, 1), 256, 0, st>>>(q, w, n, S.col0, S.a + k, S.part);
@@ -387,10 +420,10 @@ template <class View>
 static void ground_state_impl(const msb_op* op, const View& view, int64_t n, double tol, int maxit, const double* start,
                               double* g, GroundResult& out, cudaStream_t st) {
     const int grid = grid_for(n, 256, 8);
-    DevBuf<double> Q(3 * size_t(n)), v0(n), hbuf(n), part(size_t(grid) * 3), a_dev(maxit + 1), b_dev(maxit + 1),
-        bcur(1), n0(1);
+    const int part_n = std::max(3 * grid, 4096);
+    DevBuf<double> Q(3 * size_t(n)), v0(n), hbuf(n), part(part_n), a_dev(maxit + 1), b_dev(maxit + 1), bcur(1), n0(1);
     DevBuf<int> col0(1);
-    const GroundScratch S{Q.p, v0.p, hbuf.p, a_dev.p, b_dev.p, bcur.p, n0.p, col0.p, part.p};
+    const GroundScratch S{Q.p, v0.p, hbuf.p, a_dev.p, b_dev.p, bcur.p, n0.p, col0.p, part.p, part_n};
     lanczos_ground(op, view, n, tol, maxit, start, g, S, grid, out, st);
 }
 
@@ -1749,6 +1782,7 @@ static void ground_state_noalloc_impl(const msb_op* op, const View& view, int64_
     S.n0 = S.bcur + 1;
     S.col0 = reinterpret_cast<int*>(S.n0 + 1);
     S.part = S.n0 + 2;                        // partial sums, 3 per block
+    S.part_n = 3 * kNoAllocMaxGrid;
     lanczos_ground(op, view, n, tol, maxit, start, g, S, grid, out, st);
 }
 

@@ -41,6 +41,7 @@
 #include <cmath>
 #include <memory>
 
+#include "hubrows.cuh"
 #include "kernels.cuh"
 #include "msbicg_impl.cuh"
 #include "profile.cuh"
@@ -108,6 +109,49 @@ __global__ void __launch_bounds__(256) k_mvm_dot(View op, const V* __restrict__ 
     }
     store_partials<2>(acc, sm, part);
 }
+
+// The same as the epilogue of the row-tiled Hubbard product (hubrows.cuh).
+template <typename V>
+struct MvmEpi {
+    V* v;
+    const SeedState* st;
+    double* part;
+    const V* pt;
+    double c0i;
+    double acc[2];
+    DF4 df;
+    __device__ __forceinline__ bool stop() const { return st->done != 0; }
+    __device__ __forceinline__ void begin(int) {}
+    __device__ __forceinline__ void term(int64_t s, V ps, V vs) {
+        if constexpr (std::is_same<V, float2>::value) {
+            if (pt) her_acc_df(pt[s], vs, df);
+            else bil_acc_df(ps, vs, df);
+        } else {
+            if (pt) her_acc(pt[s], vs, acc[0], acc[1]);
+            else bil_acc(ps, vs, acc[0], acc[1]);
+        }
+    }
+    template <typename S>
+    __device__ __forceinline__ void operator()(int64_t s, V xs, V a, S dg, S mt) {
+        const V h = hub_value(a, dg, mt, S(c0i), xs);
+        v[s] = h;
+        term(s, xs, h);
+    }
+    __device__ __forceinline__ void pair(int64_t s, float2 xa, float2 xb, float2 a, float2 b, float da, float db,
+                                         float mt) {
+        const float2 p = hub_value(a, da, mt, float(c0i), xa), q = hub_value(b, db, mt, float(c0i), xb);
+        *reinterpret_cast<float4*>(v + s) = make_float4(p.x, p.y, q.x, q.y);
+        term(s, xa, p);
+        term(s + 1, xb, q);
+    }
+    __device__ __forceinline__ void finish(double* sm) {
+        if constexpr (std::is_same<V, float2>::value) {
+            acc[0] = df_value(df.rh, df.rl);
+            acc[1] = df_value(df.ih, df.il);
+        }
+        store_partials<2>(acc, sm, part);
+    }
+};
 
 // Dual-space product v~ = (A + c0*) p~ = (A + c0)^dagger p~ for Hermitian A (App. A).
 template <class View, typename V>
@@ -529,7 +573,9 @@ struct SolverImpl {
     using C = V;
     const SolveProblem& pr;
     cudaStream_t st;
-    int nslot, B, grid_vec, grid_flush;
+    int nslot, B, grid_vec, grid_flush, grid_mvm;
+    RowPlan rows;                 // row-tiled seed product (Hubbard without a second amplitude or phases)
+    const HubPart* rparts = nullptr;
     DevBuf<V> ring, p, v, Pbuf;
     DevBuf<V> rt, pt, vt;     // dual-space vectors (App. A), allocated only for the dual form
     DevBuf<double> part;
@@ -554,11 +600,15 @@ struct SolverImpl {
         const double nb = double(n) * csz;
         {
             ProfScope ps("seed_mvm", st, 2 * nb + op->matrix_bytes(csz), op->hx_flops() + 16.0 * n);
-            k_mvm_dot<View, V><<<grid_vec, 256, 0, st>>>(view, p.p, v.p, n, pr.c0.x, pr.c0.y, state.p, part.p, pt.p);
+            if (rows.ok)
+                launch_hub_rows<V>(rows, rparts, p.p, n, 1, pr.c0.x,
+                                   MvmEpi<V>{v.p, state.p, part.p, pt.p, pr.c0.y, {0.0, 0.0}, {}}, st);
+            else
+                k_mvm_dot<View, V><<<grid_vec, 256, 0, st>>>(view, p.p, v.p, n, pr.c0.x, pr.c0.y, state.p, part.p, pt.p);
         }
         {
             ProfScope ps("shift_scalars", st, 0, 0);
-            k_scalar_a<C><<<1, kScalarThreads, 0, st>>>(state.p, part.p, grid_vec, sh, pr.ns, B);
+            k_scalar_a<C><<<1, kScalarThreads, 0, st>>>(state.p, part.p, grid_mvm, sh, pr.ns, B);
         }
         if (pr.dual) {
             ProfScope ps("seed_mvm", st, 2 * nb + op->matrix_bytes(csz), op->hx_flops() + 8.0 * n);
@@ -611,12 +661,16 @@ struct SolverImpl {
         nslot = B + 1;
         grid_vec = grid_for(n, 256, 8);
         grid_flush = grid_for(pr.n_out, 256, 8);
+        constexpr bool f32 = std::is_same<V, float2>::value;
+        rows = op->kind == 2 ? (f32 ? op->plan32 : op->plan64) : row_plan<V>(op, 1);
+        if (op->kind == 2) rparts = f32 ? op->parts32.p : op->parts64.p;
+        grid_mvm = rows.ok ? rows.grid : grid_vec;
         ring.alloc(size_t(nslot) * n);
         p.alloc(n);
         v.alloc(n);
         if (pr.dual) { rt.alloc(n); pt.alloc(n); vt.alloc(n); }
         Pbuf.alloc(size_t(ns) * pr.n_out);
-        part.alloc(size_t(grid_vec) * 4);
+        part.alloc(size_t(std::max(grid_vec, grid_mvm)) * 4);
         state.alloc(1);
         zeta.alloc(ns); zeta_prev.alloc(ns); shift.alloc(ns);
         coef64.alloc(size_t(ns) * B * 2);

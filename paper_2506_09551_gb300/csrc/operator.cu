@@ -3,6 +3,7 @@
 #include <memory>
 
 #include "operator.cuh"
+#include "hubrows.cuh"
 #include "kernels.cuh"
 #include "profile.cuh"
 
@@ -66,6 +67,13 @@ static void build_hubbard(msb_op* op, const msb_model& m, int intermediate) {
     op->ndn.alloc(cd.size()); op->ndn.upload(cd.data(), cd.size());
     op->sup.alloc(op->host_up.size()); op->sup.upload(op->host_up.data(), op->host_up.size());
     op->sdn.alloc(op->host_dn.size()); op->sdn.upload(op->host_dn.data(), op->host_dn.size());
+    if (op->host_dn.size() < 32767) {
+        // rank-order copy of the down table with 16-bit entries for the row-tiled products
+        const uint16_t none = uint16_t(op->host_dn.size() << 1);
+        std::vector<uint16_t> r16(td.size());
+        for (size_t i = 0; i < td.size(); ++i) r16[i] = td[i] < 0 ? none : uint16_t(td[i]);
+        op->hdnr16.alloc(r16.size()); op->hdnr16.upload(r16.data(), r16.size());
+    }
     if (op->host_dn.size() < 32768) {
         // position-indexed copies for the continued fraction's row order
         const int64_t D = int64_t(op->host_dn.size());
@@ -119,6 +127,7 @@ static void build_hubbard(msb_op* op, const msb_model& m, int intermediate) {
     h.hdn16 = op->hdn16.p;
     h.hdn16p = op->hdn16p.p;
     h.slot16 = op->slot16.p;
+    h.hdnr16 = op->hdnr16.p;
     h.sup = op->sup.p; h.sdn = op->sdn.p;
     {
         bool un = false, dn = false;
@@ -187,6 +196,11 @@ static void build_sum(msb_op* op, const msb_op* const* ops, const double* shifts
     }
     for (int i = n; i <= kMaxParts; ++i) v.off[i] = off;
     op->dim = off;
+    op->plan64 = row_plan<double2>(op, 1);
+    op->plan32 = row_plan<float2>(op, 1);
+    if (op->plan64.ok) { op->parts64.alloc(n); op->parts64.upload(op->plan64.parts.data(), n); }
+    if (op->plan32.ok) { op->parts32.alloc(n); op->parts32.upload(op->plan32.parts.data(), n); }
+    MSB_CUDA(cudaDeviceSynchronize());
 }
 
 // ---------------------------------------------------------------------------
@@ -203,6 +217,42 @@ __global__ void __launch_bounds__(256) k_apply(View op, const V* __restrict__ x,
         const V h = op.hx(s, xc, xs);
         yc[s] = vadd(h, cscale(c0r, c0i, xs));
     }
+}
+
+// Epilogue of the row-tiled product (hubrows.cuh): y = (A + c0) x.
+template <typename V>
+struct ApplyEpi {
+    V* y;
+    int64_t n;
+    double c0i;
+    __device__ __forceinline__ bool stop() const { return false; }
+    __device__ __forceinline__ void begin(int col) { y += int64_t(col) * n; }
+    template <typename S>
+    __device__ __forceinline__ void operator()(int64_t s, V xs, V acc, S dg, S mt) {
+        y[s] = hub_value(acc, dg, mt, S(c0i), xs);
+    }
+    __device__ __forceinline__ void pair(int64_t s, float2 xa, float2 xb, float2 a, float2 b, float da, float db,
+                                         float mt) {
+        const float2 p = hub_value(a, da, mt, float(c0i), xa), q = hub_value(b, db, mt, float(c0i), xb);
+        *reinterpret_cast<float4*>(y + s) = make_float4(p.x, p.y, q.x, q.y);
+    }
+    __device__ __forceinline__ void finish(double*) const {}
+};
+
+template <typename V>
+static bool launch_apply_rows(const msb_op* op, double2 c0, const void* x, void* y, int nvec, cudaStream_t st) {
+    const bool f32 = std::is_same<V, float2>::value;
+    const RowPlan p = op->kind == 2 ? (f32 ? op->plan32 : op->plan64) : row_plan<V>(op, nvec);
+    if (!p.ok) return false;
+    // two adjacent FP32 elements move as 16 bytes: every vector must start on that boundary
+    if (p.pair && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u)) return false;
+    const int64_t n = op->dim;
+    ProfScope ps("h_apply", st, nvec * 2.0 * n * sizeof(V), nvec * (op->hx_flops() + 8.0 * n));
+    launch_hub_rows<V>(p, op->kind == 2 ? (f32 ? op->parts32.p : op->parts64.p) : nullptr, (const V*)x, n, nvec, c0.x,
+                       ApplyEpi<V>{(V*)y, n, c0.y}, st);
+    MSB_LAUNCH_CHECK();
+    count_launch();
+    return true;
 }
 
 template <class View>
@@ -225,6 +275,11 @@ void op_apply(msb_op* op, double2 c0, const void* x, void* y, int nvec, msb_prec
     MSB_REQUIRE(x != nullptr && y != nullptr, "x / y is NULL");
     MSB_REQUIRE(nvec >= 1 && nvec <= 65535, "nvec must be in 1..65535");
     MSB_REQUIRE(prec == MSB_FP64 || prec == MSB_FP32_MIXED, "unknown precision");
+    if (op->kind != 1 && (prec == MSB_FP64 ? launch_apply_rows<double2>(op, c0, x, y, nvec, st)
+                                           : launch_apply_rows<float2>(op, c0, x, y, nvec, st))) {
+        prof_collect();
+        return;
+    }
     if (op->kind == 0) launch_apply(op, op->hub, op->dim, c0, x, y, nvec, prec, st);
     else if (op->kind == 1) launch_apply(op, op->csr, op->dim, c0, x, y, nvec, prec, st);
     else launch_apply(op, op->sum, op->dim, c0, x, y, nvec, prec, st);

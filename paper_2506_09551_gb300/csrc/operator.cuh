@@ -40,6 +40,22 @@ __device__ __forceinline__ float vscale(float a, float v) { return a * v; }
 __device__ __forceinline__ double2 vscale(double a, double2 v) { return make_double2(a * v.x, a * v.y); }
 __device__ __forceinline__ float2 vscale(float a, float2 v) { return make_float2(a * v.x, a * v.y); }
 
+// acc + v, or acc - v when bit 0 of the table entry h is set.  One FMA per component
+// with a multiplier +-1 built in the integer pipe: selecting between an add and a
+// subtract compiles to both, predicated, and a predicated-off FP64 instruction still
+// holds the FP64 pipe (the pipe that bounds every FP64 product here).
+__device__ __forceinline__ double hop_sign(double, int32_t h) { return __hiloint2double(0x3FF00000 | (h << 31), 0); }
+__device__ __forceinline__ float hop_sign(float, int32_t h) { return __int_as_float(0x3F800000 | (h << 31)); }
+__device__ __forceinline__ double vhop(double acc, int32_t h, double v) { return fma(hop_sign(0.0, h), v, acc); }
+__device__ __forceinline__ double2 vhop(double2 acc, int32_t h, double2 v) {
+    const double g = hop_sign(0.0, h);
+    return make_double2(fma(g, v.x, acc.x), fma(g, v.y, acc.y));
+}
+__device__ __forceinline__ float2 vhop(float2 acc, int32_t h, float2 v) {
+    const float g = hop_sign(0.f, h);
+    return make_float2(fmaf(g, v.x, acc.x), fmaf(g, v.y, acc.y));
+}
+
 template <typename V> struct Scalar;
 template <> struct Scalar<double> { using type = double; };
 template <> struct Scalar<float> { using type = float; };
@@ -73,6 +89,8 @@ struct HubView {
                             // empty slots hold Ddn << 1 (index Ddn: a zero kept past the staged row)
     const uint16_t* hdn16p; // the same with targets moved to their shared-memory slots (FP32 apply), or null
     const uint16_t* slot16; // shared-memory slot of each position (with hdn16p), or null
+    const uint16_t* hdnr16; // [slot][state] down-spin table in rank order, entries (target rank << 1) | neg;
+                            // empty slots hold Ddn << 1 (Ddn < 32767, else null)
     const uint32_t* sup;   // occupation strings, rank order
     const uint32_t* sdn;
     int usign, dsign;      // 1 if some up / down hop carries a negative sign (Jordan-Wigner string)
@@ -140,14 +158,14 @@ struct HubView {
         for (int e = 0; e < nu; ++e) {
             const int32_t h = __ldg(hup + int64_t(e) * Dup + iu);
             const V v = x[int64_t(h >> 1) * Ddn + id];
-            acc = (h & 1) ? vsub(acc, v) : vadd(acc, v);
+            acc = vhop(acc, h, v);
         }
         const int nd = __ldg(ndn + id);
         const V* __restrict__ xrow = x + iu * Ddn;
         for (int e = 0; e < nd; ++e) {
             const int32_t h = __ldg(hdn + int64_t(e) * Ddn + id);
             const V v = xrow[h >> 1];
-            acc = (h & 1) ? vsub(acc, v) : vadd(acc, v);
+            acc = vhop(acc, h, v);
         }
         // H x = diag * x - t * sum(sign * x_neighbour) - t2 * sum over the diagonal bonds
         V out = vaxpy(S(-t), acc, vscale(diag<S>(iu, id), xs));
@@ -157,13 +175,13 @@ struct HubView {
             for (int e = 0; e < nu2; ++e) {
                 const int32_t h = __ldg(hup2 + int64_t(e) * Dup + iu);
                 const V v = x[int64_t(h >> 1) * Ddn + id];
-                acc2 = (h & 1) ? vsub(acc2, v) : vadd(acc2, v);
+                acc2 = vhop(acc2, h, v);
             }
             const int nd2 = __ldg(ndn2 + id);
             for (int e = 0; e < nd2; ++e) {
                 const int32_t h = __ldg(hdn2 + int64_t(e) * Ddn + id);
                 const V v = xrow[h >> 1];
-                acc2 = (h & 1) ? vsub(acc2, v) : vadd(acc2, v);
+                acc2 = vhop(acc2, h, v);
             }
             out = vaxpy(S(-t2), acc2, out);
         }
@@ -172,7 +190,8 @@ struct HubView {
 
     template <typename V>
     __device__ __forceinline__ V hx(int64_t s, const V* __restrict__ x, V xs) const {
-        const int64_t iu = s / Ddn, id = s - iu * Ddn;
+        const uint32_t iu = uint32_t(s) / uint32_t(Ddn);      // s < D_up D_dn < 2^32 for L <= 16
+        const int64_t id = s - int64_t(iu) * Ddn;
         return hx_at(iu, id, x, xs);
     }
 };
@@ -243,6 +262,33 @@ struct CsrView {
 
 }  // namespace msb
 
+namespace msb {
+
+// One Hubbard block of a row-tiled product (hubrows.cuh): its view, the offset of its
+// part of the vector, the diagonal shift, and its tiles (first tile, rows per tile,
+// parts per row).
+struct HubPart {
+    HubView v;
+    int64_t off;
+    double shift;
+    int tile0, R, split;
+};
+
+// Tiles and launch shape of a row-tiled product.
+struct RowPlan {
+    bool ok = false;
+    int threads = 0;
+    int np = 0;               // parts
+    int64_t tiles = 0;
+    int grid = 0;             // CTAs per column (each loops over tiles when tiles > grid)
+    size_t smem = 0;
+    bool pair = false;        // FP32: every D_dn even, two elements per thread
+    HubPart one{};            // the part of a single operator (passed by value)
+    std::vector<HubPart> parts;
+};
+
+}  // namespace msb
+
 // ----------------------------------------------------------------------------
 // Library-side operator object (host).
 // ----------------------------------------------------------------------------
@@ -256,7 +302,7 @@ struct msb_op {
     msb::DevBuf<int32_t> hup, hdn, hup2, hdn2;
     msb::DevBuf<uint8_t> dirup, dirdn;
     msb::DevBuf<uint8_t> nup, ndn, nup2, ndn2;
-    msb::DevBuf<uint16_t> hdn16, hdn16p, slot16, dpos;
+    msb::DevBuf<uint16_t> hdn16, hdn16p, slot16, dpos, hdnr16;
     msb::DevBuf<uint8_t> ndnp;
     msb::DevBuf<uint32_t> sdnp;
     msb::DevBuf<uint32_t> sup, sdn;
@@ -271,6 +317,8 @@ struct msb_op {
     // direct sum (parts are not owned: the caller keeps them alive)
     std::vector<const msb_op*> parts;
     msb::SumView sum{};
+    msb::RowPlan plan64, plan32;             // row-tiled product of the sum (FP64, FP32 vectors)
+    msb::DevBuf<msb::HubPart> parts64, parts32;
     int device = 0;
     double offdiag = 0;          // off-diagonal entries (hops, or CSR nonzeros)
     double offdiag2 = 0;         // of them, the diagonal-bond hops of a 2D cluster
