@@ -44,8 +44,9 @@ __device__ __forceinline__ void hop_add(float4& a, float g, float4 v) {
     a.x = fmaf(g, v.x, a.x); a.y = fmaf(g, v.y, a.y); a.z = fmaf(g, v.z, a.z); a.w = fmaf(g, v.w, a.w);
 }
 
-// Epi: operator()(s, xs, acc, dg, mt): element s of the column, x[s], the signed hop
-// sum, the diagonal (shift and c0r included) and -t; finish(tile partial store).
+// Epi: operator()(s, xs, acc, dg, mt, shift): element s of the column, x[s], the signed
+// hop sum, the diagonal, -t and the block's shift (hub_value forms H x + c0 x from them);
+// finish(): partial sums.
 // PAIR (float2, even D_dn): two adjacent elements per thread.
 template <typename V, bool Multi, bool PAIR, class Epi>
 __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __restrict__ parts, int np,
@@ -54,7 +55,7 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
     using S = scalar_t<V>;
     if (epi.stop()) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    __shared__ double red[64];
+    __shared__ double red[2 * 256];
     const int nt = blockDim.x;
     epi.begin(blockIdx.y);
     const V* __restrict__ xc = x + int64_t(blockIdx.y) * ldx;
@@ -117,7 +118,11 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
         }
         for (int i = threadIdx.x; i < 3 * (L + 1); i += nt) {
             const int nb = i / (L + 1), pc = i - nb * (L + 1);
-            lut[i] = S(h.U * double(pc) - h.Uc * double(nb) + P.shift + c0r);
+            // FP64: c0's real part and the block's shift are folded into the diagonal, which saves
+            // two FP64 operations per element at the same rounding error.  FP32: they stay
+            // apart, since the sum rounded to 32 bits would perturb the operator.
+            if constexpr (sizeof(S) == 8) lut[i] = h.U * double(pc) - h.Uc * double(nb) + P.shift + c0r;
+            else lut[i] = h.Uf * float(pc) - h.Ucf * float(nb);
         }
         __syncthreads();
         const int core = h.core;
@@ -180,7 +185,7 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
                 const float da = lut[__popc(su & sa) + na * (L + 1)], db = lut[__popc(su & sb) + nb * (L + 1)];
                 if (act) {
                     const float2 xa = xr[d], xb = xr[d + 1];
-                    epi.pair(base + e, xa, xb, make_float2(a.x, a.y), make_float2(a.z, a.w), da, db, mt);
+                    epi.pair(base + e, xa, xb, make_float2(a.x, a.y), make_float2(a.z, a.w), da, db, mt, float(P.shift));
                 }
             } else {
                 V a = vzero(V{});
@@ -208,7 +213,7 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
                 const uint32_t sd = __ldg(h.sdn + d);
                 const int nb = core >= 0 ? int((su >> core) & 1u) + int((sd >> core) & 1u) : 0;
                 const S dg = lut[__popc(su & sd) + nb * (L + 1)];
-                if (act) epi(base + e, xr[d], a, dg, mt);
+                if (act) epi(base + e, xr[d], a, dg, mt, S(P.shift));
             }
         }
         __syncthreads();                                           // the tile's shared memory is reused
@@ -216,12 +221,17 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
     epi.finish(red);
 }
 
-// H x + c0 x from the hop sum and the diagonal (c0's real part already in dg).
-__device__ __forceinline__ double2 hub_value(double2 acc, double dg, double mt, double c0i, double2 x) {
+// H x + c0 x from the hop sum and the diagonal.  FP64: the real part of c0 and the shift
+// are in dg.  FP32: added here, in the order of the element-wise kernels.
+__device__ __forceinline__ double2 hub_value(double2 acc, double dg, double mt, double, double, double c0i, double2 x) {
     return make_double2(fma(mt, acc.x, fma(dg, x.x, -c0i * x.y)), fma(mt, acc.y, fma(dg, x.y, c0i * x.x)));
 }
-__device__ __forceinline__ float2 hub_value(float2 acc, float dg, float mt, float c0i, float2 x) {
-    return make_float2(fmaf(mt, acc.x, fmaf(dg, x.x, -c0i * x.y)), fmaf(mt, acc.y, fmaf(dg, x.y, c0i * x.x)));
+__device__ __forceinline__ float2 hub_value(float2 acc, float dg, float mt, float shift, double c0r, double c0i,
+                                            float2 x) {
+    float2 h = make_float2(__fmaf_rn(mt, acc.x, __fmul_rn(dg, x.x)), __fmaf_rn(mt, acc.y, __fmul_rn(dg, x.y)));
+    if (shift != 0.f) h = vaxpy(shift, x, h);
+    const float2 c = cscale_rn(float(c0r), float(c0i), x);
+    return make_float2(__fadd_rn(h.x, c.x), __fadd_rn(h.y, c.y));
 }
 
 // Tiles of an operator's blocks and the launch shape for vectors of element V with

@@ -16,6 +16,11 @@ __device__ __forceinline__ float2 cscale(double cr, double ci, float2 v) {
     const float a = float(cr), b = float(ci);
     return make_float2(a * v.x - b * v.y, a * v.y + b * v.x);
 }
+// The FP32 product with its rounding written out (one multiplication, one FMA per part),
+// so that every kernel that uses it rounds alike whatever the code around it.
+__device__ __forceinline__ float2 cscale_rn(float a, float b, float2 v) {
+    return make_float2(__fmaf_rn(a, v.x, -__fmul_rn(b, v.y)), __fmaf_rn(b, v.x, __fmul_rn(a, v.y)));
+}
 __device__ __forceinline__ double cscale(double cr, double, double v) { return cr * v; }
 __device__ __forceinline__ float cscale(double cr, double, float v) { return float(cr) * v; }
 
@@ -135,6 +140,54 @@ __device__ __forceinline__ void store_partials(double (&v)[NV], double* sm, doub
 #pragma unroll
         for (int i = 0; i < NV; ++i) part[base + i] = v[i];
     }
+}
+
+// Block sum of NV doubles per thread in thread 0, through shared memory: one warp adds
+// the other warps' values lane by lane and then shuffles, (threads / 32 + 5) NV FP64
+// additions per CTA where a shuffle tree in every warp takes 5 NV per warp (the FP64
+// pipe spends 16 cycles on a warp's addition).  sm: NV * blockDim.x doubles.
+template <int NV>
+__device__ __forceinline__ void block_sum_sm(double (&v)[NV], double* sm) {
+    const int nt = blockDim.x;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) sm[i * nt + threadIdx.x] = v[i];
+    __syncthreads();
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+            for (int t = threadIdx.x + 32; t < nt; t += 32) v[i] += sm[i * nt + t];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
+    }
+    __syncthreads();
+}
+
+// True in every thread of the last CTA to arrive among `total`, once all their global
+// writes before this call are visible to it.  The counter returns to zero.  Every
+// thread of the CTA must call it.
+__device__ __forceinline__ bool last_cta(unsigned* counter, int total) {
+    __shared__ int s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicInc(counter, unsigned(total - 1)) == unsigned(total - 1);
+        __threadfence();
+    }
+    __syncthreads();
+    return s_last != 0;
+}
+
+// Sum of n x NV partials written by other CTAs of this launch (read past L1), in a fixed
+// order; thread 0.  sm: NV * blockDim.x doubles.
+template <int NV>
+__device__ __forceinline__ void sum_partials_cg(const double* part, int n, double (&v)[NV], double* sm) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = 0.0;
+    for (int b = threadIdx.x; b < n; b += blockDim.x) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] += __ldcg(part + int64_t(b) * NV + i);
+    }
+    block_sum_sm<NV>(v, sm);
 }
 
 // CUDA device sanity check used by every compute entry point.

@@ -143,16 +143,17 @@ struct LzEpi {
     double bp, dot;
     __device__ __forceinline__ bool stop() const { return false; }
     __device__ __forceinline__ void begin(int) { bp = bprev[0]; }
-    __device__ __forceinline__ void operator()(int64_t s, double xs, double acc, double dg, double mt) {
+    __device__ __forceinline__ void operator()(int64_t s, double xs, double acc, double dg, double mt, double) {
         double h = fma(mt, acc, dg * xs);
         if (bp != 0.0) h = fma(-bp, qp[s], h);
         w[s] = h;
         dot = fma(xs, h, dot);
     }
-    __device__ __forceinline__ void pair(int64_t, float2, float2, float2, float2, float, float, float) {}
+    __device__ __forceinline__ void pair(int64_t, float2, float2, float2, float2, float, float, float, float) {}
     __device__ __forceinline__ void finish(double* sm) {
         double acc[1] = {dot};
-        store_partials<1>(acc, sm, part);
+        block_sum_sm<1>(acc, sm);
+        if (threadIdx.x == 0) part[blockIdx.x] = acc[0];
     }
 };
 

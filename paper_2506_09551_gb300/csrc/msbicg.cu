@@ -49,6 +49,7 @@
 namespace msb {
 
 constexpr int kScalarThreads = 256;
+constexpr int kVecThreads = 512;      // vector kernels of the iteration, two CTAs per SM
 
 // ---------------------------------------------------------------------------
 // Device state
@@ -58,14 +59,22 @@ struct SeedState {
     double2 alpha;        // alpha_m of the current iteration
     double2 alpha_prev;   // alpha_{m-1} (1 before the first iteration)
     double2 beta;         // beta_m: built p_m (0 at m = 0)
+    double2 beta_n, rho_n;   // beta_{m+1}, (r~_{m+1}, r~_{m+1}) before the rescale
+    double rn_n;          // ||r~_{m+1}||
+    int f_n, bad_n;       // its rescale exponent; why beta could not be formed
+    unsigned cnt_a, cnt_b;   // arrival counters of the two reductions
     double rnorm;         // ||r_m||
     double bnorm;         // ||b||
+    double ibnorm;        // 1 / ||b|| (0 for b = 0)
     double tol;
     int m;                // iteration count
     int m0;               // iteration at the start of the current block
     int j;                // iterations in the current block
-    int slot;             // ring slot holding r_m
-    int done;
+    int jcur;             // j at the start of the iteration
+    int slot0;            // ring slot holding r_{m0}
+    int stop;             // the recurrence ended (set by k_update_p)
+    int halted;           // copy of `stop` made by the product kernel, read by the two after it
+    int bad;              // alpha could not be formed
     int status;           // msb_status of the recurrence
     int maxit;
     int nactive;
@@ -75,18 +84,80 @@ struct SeedState {
 };
 
 // ---------------------------------------------------------------------------
-// Kernels of one iteration.  All of them return at once once state->done.
+// One iteration is three launches (four in the dual form), since the sums that alpha
+// and beta need close over the whole vector:
+//   the product      v = A p; its last CTA to finish: mu, alpha
+//   k_seed_update    r_{m+1} = r_m - alpha v; its last CTA: rho, the norm, beta
+//   k_update_p       p_{m+1} = r_{m+1} + beta p_m
+// CTA 0 of the two vector kernels does the per-shift scalars meanwhile.  A kernel never
+// writes a state field that its other CTAs read (`halted`, `jcur`, `beta_n` and the
+// like are written one launch before they are read).  After the recurrence has ended
+// all of them return at once.  FP64 scalar work is left to one thread or one warp: the
+// FP64 pipe spends 16 cycles on a warp's instruction, so a division by every warp of
+// every CTA costs more than the vectors (measured: alpha and beta formed by each CTA,
+// 85 us for the two vector kernels at L = 12, as much as with separate scalar kernels).
 // ---------------------------------------------------------------------------
+
+// a / b with one division: b scaled by an exact power of two, so that |b|^2 lies in [1, 8).
+__device__ __forceinline__ double2 cdiv1(double2 a, double2 b) {
+    const unsigned ex = unsigned(__double2hiint(b.x) >> 20) & 0x7FFu, ey = unsigned(__double2hiint(b.y) >> 20) & 0x7FFu;
+    const unsigned e = max(ex, ey);
+    if (e == 0u || e >= 0x7FEu) return cdiv(a, b);           // zero, subnormal, at the top of the range, not finite
+    const double s = __hiloint2double(int((0x7FEu - e) << 20), 0);         // 2^(1023 - e)
+    const double bx = b.x * s, by = b.y * s;
+    const double r = 1.0 / fma(bx, bx, by * by) * s;
+    return make_double2(fma(a.x, bx, a.y * by) * r, fma(a.y, bx, -a.x * by) * r);
+}
+// x 2^n, exact while the result is a normal number.
+__device__ __forceinline__ double scale2(double x, int n) {
+    return n > -1022 && n < 1023 ? x * __hiloint2double((1023 + n) << 20, 0) : ldexp(x, n);
+}
+__device__ __forceinline__ double2 scale2(double2 v, int n) { return make_double2(scale2(v.x, n), scale2(v.y, n)); }
+
+// First thread block of the product kernel: the iteration's copy of `stop`.
+__device__ __forceinline__ bool mvm_halted(SeedState* st) {
+    const int h = st->stop;
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->halted = h;
+    return h != 0;
+}
+
+// End of the product kernel: partial mu, and alpha_m from all of them in the last CTA.
+// sm: 2 * blockDim.x doubles.
+__device__ __forceinline__ void mvm_finish(double (&acc)[2], double* sm, double* part, SeedState* st) {
+    block_sum_sm<2>(acc, sm);
+    if (threadIdx.x == 0) {
+        part[2 * int64_t(blockIdx.x)] = acc[0];
+        part[2 * int64_t(blockIdx.x) + 1] = acc[1];
+    }
+    if (!last_cta(&st->cnt_a, gridDim.x)) return;
+    double mu[2];
+    sum_partials_cg<2>(part, gridDim.x, mu, sm);
+    if (threadIdx.x == 0) {
+        const double2 m2 = make_double2(mu[0], mu[1]);
+        int bad = MSB_OK;
+        double2 a = make_double2(0.0, 0.0);
+        if (!cfinite(m2)) bad = MSB_ENONFINITE;
+        else if (m2.x == 0.0 && m2.y == 0.0) bad = MSB_EBREAKDOWN;
+        else {
+            a = cdiv1(st->rho, m2);
+            if (!cfinite(a)) bad = MSB_ENONFINITE;
+        }
+        if (bad) st->status = bad;
+        st->bad = bad;
+        st->alpha = a;
+        st->jcur = st->j;
+    }
+}
 
 // v = A p (A = op + c0), partial mu = (p, v).
 // Dual form (pt != null, App. A): mu = <p~|v> (Hermitian) instead of (p, v).
 template <class View, typename V>
 __global__ void __launch_bounds__(256) k_mvm_dot(View op, const V* __restrict__ p, V* __restrict__ v,
                                                  int64_t n, double c0r, double c0i,
-                                                 const SeedState* __restrict__ st, double* part,
+                                                 SeedState* __restrict__ st, double* part,
                                                  const V* __restrict__ pt) {
-    if (st->done) return;
-    __shared__ double sm[2 * 32];
+    if (mvm_halted(st)) return;
+    __shared__ double sm[2 * 256];
     double acc[2] = {0.0, 0.0};
     DF4 df;
     for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n;
@@ -107,20 +178,20 @@ __global__ void __launch_bounds__(256) k_mvm_dot(View op, const V* __restrict__ 
         acc[0] = df_value(df.rh, df.rl);
         acc[1] = df_value(df.ih, df.il);
     }
-    store_partials<2>(acc, sm, part);
+    mvm_finish(acc, sm, part, st);
 }
 
 // The same as the epilogue of the row-tiled Hubbard product (hubrows.cuh).
 template <typename V>
 struct MvmEpi {
     V* v;
-    const SeedState* st;
+    SeedState* st;
     double* part;
     const V* pt;
-    double c0i;
+    double c0r, c0i;
     double acc[2];
     DF4 df;
-    __device__ __forceinline__ bool stop() const { return st->done != 0; }
+    __device__ __forceinline__ bool stop() const { return mvm_halted(st); }
     __device__ __forceinline__ void begin(int) {}
     __device__ __forceinline__ void term(int64_t s, V ps, V vs) {
         if constexpr (std::is_same<V, float2>::value) {
@@ -132,14 +203,14 @@ struct MvmEpi {
         }
     }
     template <typename S>
-    __device__ __forceinline__ void operator()(int64_t s, V xs, V a, S dg, S mt) {
-        const V h = hub_value(a, dg, mt, S(c0i), xs);
+    __device__ __forceinline__ void operator()(int64_t s, V xs, V a, S dg, S mt, S shift) {
+        const V h = hub_value(a, dg, mt, shift, c0r, c0i, xs);
         v[s] = h;
         term(s, xs, h);
     }
     __device__ __forceinline__ void pair(int64_t s, float2 xa, float2 xb, float2 a, float2 b, float da, float db,
-                                         float mt) {
-        const float2 p = hub_value(a, da, mt, float(c0i), xa), q = hub_value(b, db, mt, float(c0i), xb);
+                                         float mt, float shift) {
+        const float2 p = hub_value(a, da, mt, shift, c0r, c0i, xa), q = hub_value(b, db, mt, shift, c0r, c0i, xb);
         *reinterpret_cast<float4*>(v + s) = make_float4(p.x, p.y, q.x, q.y);
         term(s, xa, p);
         term(s + 1, xb, q);
@@ -149,7 +220,7 @@ struct MvmEpi {
             acc[0] = df_value(df.rh, df.rl);
             acc[1] = df_value(df.ih, df.il);
         }
-        store_partials<2>(acc, sm, part);
+        mvm_finish(acc, sm, part, st);
     }
 };
 
@@ -157,47 +228,25 @@ struct MvmEpi {
 template <class View, typename V>
 __global__ void __launch_bounds__(256) k_dual_mvm(View op, const V* __restrict__ pt, V* __restrict__ vt, int64_t n,
                                                   double c0r, double c0i, const SeedState* __restrict__ st) {
-    if (st->done) return;
+    if (st->halted) return;
     for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n; s += int64_t(gridDim.x) * blockDim.x) {
         const V ps = pt[s];
         vt[s] = vadd(op.hx(s, pt, ps), cscale(c0r, -c0i, ps));
     }
 }
 
-// alpha, and every active shift's zeta / gamma / c for block position j.
+// Every active shift's zeta / gamma / c for block position j (one CTA).
 template <typename C>
-__global__ void __launch_bounds__(kScalarThreads) k_scalar_a(SeedState* st, const double* part, int nblk,
-                                                             ShiftArrays sh, int ns, int B) {
-    if (st->done) return;
-    __shared__ double sm[2 * 32];
-    __shared__ double2 s_alpha;
-    __shared__ int s_bad;
-    double mu[2];
-    reduce_partials<2>(part, nblk, mu, sm);
-    if (threadIdx.x == 0) {
-        const double2 m2 = make_double2(mu[0], mu[1]);
-        s_bad = 0;
-        if (!cfinite(m2)) {
-            st->status = MSB_ENONFINITE; st->done = 1; s_bad = 1;
-        } else if (m2.x == 0.0 && m2.y == 0.0) {
-            st->status = MSB_EBREAKDOWN; st->done = 1; s_bad = 1;
-        } else {
-            const double2 a = cdiv(st->rho, m2);
-            if (!cfinite(a)) { st->status = MSB_ENONFINITE; st->done = 1; s_bad = 1; }
-            st->alpha = a;
-            s_alpha = a;
-        }
-    }
-    __syncthreads();
-    if (s_bad) return;
-    const double2 alpha = s_alpha;
+__device__ __forceinline__ void shift_scalars_a(SeedState* st, double2 alpha, const ShiftArrays& sh, int ns, int B) {
+    if (threadIdx.x >= ns) return;
     const double2 beta = st->beta;
-    const double2 ab_over = cdiv(cmul(alpha, beta), st->alpha_prev);   // alpha_m beta_m / alpha_{m-1}
+    const double2 ab_over = cdiv1(cmul(alpha, beta), st->alpha_prev);   // alpha_m beta_m / alpha_{m-1}
     const int j = st->j;
     const int fexp = st->fexp;
     for (int k = threadIdx.x; k < ns; k += blockDim.x) {
         if (!sh.active[k]) continue;
         const double2 z = sh.zeta[k], zp = sh.zeta_prev[k], s = sh.shift[k];
+        const int ze = sh.zexp[k];
         // (1 - alpha s) z + (alpha beta / alpha_prev)(z - zp)
         const double2 one_m = make_double2(1.0 - (alpha.x * s.x - alpha.y * s.y), -(alpha.x * s.y + alpha.y * s.x));
         const double2 zn = cadd(cmul(one_m, z), cmul(ab_over, csub(z, zp)));
@@ -208,11 +257,10 @@ __global__ void __launch_bounds__(kScalarThreads) k_scalar_a(SeedState* st, cons
             continue;
         }
         // beta_m zeta_{m-1} / zeta_m, times S_m / S_{m-1}
-        double2 gamma = cdiv(cmul(beta, zp), z);
-        gamma = make_double2(ldexp(gamma.x, fexp), ldexp(gamma.y, fexp));
+        const double2 gamma = scale2(cmul(cmul(beta, zp), sh.izeta[k]), fexp);
         // alpha_m / zeta_{m+1} / S_m
-        double2 c = cdiv(alpha, zn);
-        c = make_double2(ldexp(c.x, sh.zexp[k]), ldexp(c.y, sh.zexp[k]));
+        const double2 izn = cdiv1(make_double2(1.0, 0.0), zn);
+        const double2 c = scale2(cmul(alpha, izn), ze);
         const int64_t o = int64_t(k) * B + j;
         sh.coef64[2 * o] = gamma;
         sh.coef64[2 * o + 1] = c;
@@ -223,31 +271,72 @@ __global__ void __launch_bounds__(kScalarThreads) k_scalar_a(SeedState* st, cons
         const double mag = fmax(fabs(zn.x), fabs(zn.y));
         int q = 0;
         if (mag < 0x1p-30 || mag > 0x1p30) q = -ilogb(mag);
-        sh.zeta_prev[k] = make_double2(ldexp(z.x, q), ldexp(z.y, q));
-        sh.zeta[k] = make_double2(ldexp(zn.x, q), ldexp(zn.y, q));
-        sh.zexp[k] += q;
+        sh.zeta_prev[k] = scale2(z, q);
+        sh.zeta[k] = scale2(zn, q);
+        sh.izeta[k] = scale2(izn, -q);
+        sh.zexp[k] = ze + q;
     }
 }
 
-// r_{m+1} = r_m - alpha v (into the next ring slot); partials (r,r), ||r||^2.
+// Sums of one residual element: x.x, y.y and x.y of its parts, from which rho =
+// (Sxx - Syy) + 2 i Sxy and ||r||^2 = Sxx + Syy follow: three products per element
+// where rho and the norm separately take six.
+struct ResSum {
+    double xx = 0.0, yy = 0.0, xy = 0.0;
+    __device__ __forceinline__ void add(double2 r) {
+        xx = fma(r.x, r.x, xx);
+        yy = fma(r.y, r.y, yy);
+        xy = fma(r.x, r.y, xy);
+    }
+    __device__ __forceinline__ void get(double (&a)[3]) const { a[0] = xx - yy; a[1] = 2.0 * xy; a[2] = xx + yy; }
+};
+struct ResSumF {
+    float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f, ch = 0.f, cl = 0.f;
+    __device__ __forceinline__ void add(float2 r) {
+        df_add_prod(xh, xl, r.x, r.x);
+        df_add_prod(yh, yl, r.y, r.y);
+        df_add_prod(ch, cl, r.x, r.y);
+    }
+    __device__ __forceinline__ void get(double (&a)[3]) const {
+        const double xx = df_value(xh, xl), yy = df_value(yh, yl);
+        a[0] = xx - yy; a[1] = 2.0 * df_value(ch, cl); a[2] = xx + yy;
+    }
+};
+template <typename V> using res_sum_t = typename std::conditional<std::is_same<V, float2>::value, ResSumF, ResSum>::type;
+
+// r + sg (c v), sg = +-1, the product rounded before it is added.
+__device__ __forceinline__ float2 axpy_rn(float2 r, float2 c, float2 v, float sg) {
+    const float2 t = cscale_rn(c.x, c.y, v);
+    return make_float2(__fmaf_rn(sg, t.x, r.x), __fmaf_rn(sg, t.y, r.y));
+}
+
+// r_{m+1} = r_m - alpha v (into the next ring slot; slots ld elements apart, ld even);
+// partials of rho and ||r||^2.  CTA 0: the per-shift scalars.
 // Dual form (rt != null): also r~ <- r~ - conj(alpha) v~, and rho = <r~|r> (Hermitian).
+// Bound by memory (three vectors; L2 while they fit); 16-byte accesses, two elements
+// per access in FP32, two accesses in flight per vector.
 template <typename V>
-__global__ void __launch_bounds__(256) k_seed_update(V* ring, const V* __restrict__ v, int64_t n, int nslot,
-                                                     const SeedState* __restrict__ st, double* part,
-                                                     V* __restrict__ rt, const V* __restrict__ vt) {
-    if (st->done) return;
-    __shared__ double sm[3 * 32];
-    const int cur = st->slot, nxt = (cur + 1) % nslot;
-    const V* __restrict__ r = ring + int64_t(cur) * n;
-    V* __restrict__ rn = ring + int64_t(nxt) * n;
+__global__ void __launch_bounds__(kVecThreads) k_seed_update(V* ring, int64_t ld, const V* __restrict__ v, int64_t n,
+                                                             int nslot, SeedState* __restrict__ st, double* part,
+                                                             V* __restrict__ rt, const V* __restrict__ vt,
+                                                             ShiftArrays sh, int ns, int B) {
+    if (st->halted || st->bad) return;
     const double2 a = st->alpha;
+    if (blockIdx.x == 0) {
+        shift_scalars_a<V>(st, a, sh, ns, B);
+        return;
+    }
+    __shared__ double sm[3 * kVecThreads];
+    const int cur = (st->slot0 + st->jcur) % nslot, nxt = (cur + 1) % nslot;
+    const V* __restrict__ r = ring + int64_t(cur) * ld;
+    V* __restrict__ rn = ring + int64_t(nxt) * ld;
+    const int64_t nth = int64_t(gridDim.x - 1) * blockDim.x, t0 = int64_t(blockIdx.x - 1) * blockDim.x + threadIdx.x;
     double acc[3] = {0.0, 0.0, 0.0};
-    DF4 df;
-    for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n;
-         s += int64_t(gridDim.x) * blockDim.x) {
-        const V x = vsub(r[s], cscale(a.x, a.y, v[s]));
-        rn[s] = x;
-        if (rt) {
+    if (rt) {
+        DF4 df;
+        for (int64_t s = t0; s < n; s += nth) {
+            const V x = vsub(r[s], cscale(a.x, a.y, v[s]));
+            rn[s] = x;
             const V y = vsub(rt[s], cscale(a.x, -a.y, vt[s]));
             rt[s] = y;
             if constexpr (std::is_same<V, float2>::value) {
@@ -257,140 +346,203 @@ __global__ void __launch_bounds__(256) k_seed_update(V* ring, const V* __restric
                 her_acc(y, x, acc[0], acc[1]);
                 acc[2] += norm2(x);
             }
-            continue;
         }
         if constexpr (std::is_same<V, float2>::value) {
-            bil_acc_df(x, x, df);
-            norm_acc_df(x, df);
-        } else {
-            bil_acc(x, x, acc[0], acc[1]);
-            acc[2] += norm2(x);
+            acc[0] = df_value(df.rh, df.rl);
+            acc[1] = df_value(df.ih, df.il);
+            acc[2] = df_value(df.nh, df.nl);
         }
-    }
-    if constexpr (std::is_same<V, float2>::value) {
-        acc[0] = df_value(df.rh, df.rl);
-        acc[1] = df_value(df.ih, df.il);
-        acc[2] = df_value(df.nh, df.nl);
-    }
-    store_partials<3>(acc, sm, part);
-}
-
-// beta, convergence of every shift, iteration bookkeeping, seed rescaling.
-// The rescale 2^f of r~_{m+1} is committed only if the solve goes on (a finished
-// solve keeps r~ as it is), so that fz_coef, the factor from the stored r~_{m+1}
-// to each tested shift's recursive residual, matches what the ring holds.
-__global__ void __launch_bounds__(kScalarThreads) k_scalar_b(SeedState* st, const double* part, int nblk,
-                                                             ShiftArrays sh, int ns, int nslot) {
-    if (st->done) return;
-    __shared__ double sm[3 * 32];
-    __shared__ double s_rn;      // ||r~_{m+1}|| (stored scale S_m)
-    __shared__ double2 s_rho;    // (r~_{m+1}, r~_{m+1}) at scale S_m
-    __shared__ int s_m, s_stop, s_f;
-    double v[3];
-    reduce_partials<3>(part, nblk, v, sm);
-    if (threadIdx.x == 0) {
-        const double2 rho_new = make_double2(v[0], v[1]);
-        const double rn = sqrt(v[2]);
-        st->slot = (st->slot + 1) % nslot;
-        st->m += 1;
-        st->j += 1;
-        st->alpha_prev = st->alpha;
-        s_stop = 0;
-        int f = 0;
-        if (!cfinite(rho_new) || !isfinite(rn)) {
-            st->status = MSB_ENONFINITE; s_stop = 1;
-        } else if (rn == 0.0) {
-            st->beta = make_double2(0.0, 0.0);        // exact solution: every shift converged
-        } else if (rho_new.x == 0.0 && rho_new.y == 0.0) {
-            st->status = MSB_EBREAKDOWN; s_stop = 1;   // (r, r) = 0 with r != 0
+    } else {
+        res_sum_t<V> sum;
+        if constexpr (std::is_same<V, float2>::value) {
+            const int64_t h = n >> 1;
+            const float2 af = from_d2<float2>(a);
+            const float4* __restrict__ r4 = reinterpret_cast<const float4*>(r);
+            const float4* __restrict__ v4 = reinterpret_cast<const float4*>(v);
+            float4* __restrict__ o4 = reinterpret_cast<float4*>(rn);
+            auto one = [&](int64_t i, float4 x, float4 w) {
+                const float2 p = axpy_rn(make_float2(x.x, x.y), af, make_float2(w.x, w.y), -1.f);
+                const float2 q = axpy_rn(make_float2(x.z, x.w), af, make_float2(w.z, w.w), -1.f);
+                o4[i] = make_float4(p.x, p.y, q.x, q.y);
+                sum.add(p);
+                sum.add(q);
+            };
+            int64_t i = t0;
+            for (; i + nth < h; i += 2 * nth) {
+                const float4 x0 = r4[i], w0 = v4[i], x1 = r4[i + nth], w1 = v4[i + nth];
+                one(i, x0, w0);
+                one(i + nth, x1, w1);
+            }
+            if (i < h) one(i, r4[i], v4[i]);
+            if ((n & 1) && t0 == 0) {
+                const float2 x = axpy_rn(r[n - 1], af, v[n - 1], -1.f);
+                rn[n - 1] = x;
+                sum.add(x);
+            }
         } else {
-            st->beta = cdiv(rho_new, st->rho);
+            const V na = make_double2(-a.x, -a.y);
+            int64_t i = t0;
+            for (; i + nth < n; i += 2 * nth) {
+                const V x0 = r[i], w0 = v[i], x1 = r[i + nth], w1 = v[i + nth];
+                const V y0 = cfma(na, w0, x0), y1 = cfma(na, w1, x1);
+                rn[i] = y0;
+                rn[i + nth] = y1;
+                sum.add(y0);
+                sum.add(y1);
+            }
+            if (i < n) {
+                const V y0 = cfma(na, v[i], r[i]);
+                rn[i] = y0;
+                sum.add(y0);
+            }
+        }
+        sum.get(acc);
+    }
+    block_sum_sm<3>(acc, sm);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) part[int64_t(blockIdx.x - 1) * 3 + i] = acc[i];
+    }
+    if (!last_cta(&st->cnt_b, gridDim.x - 1)) return;
+    sum_partials_cg<3>(part, gridDim.x - 1, acc, sm);
+    if (threadIdx.x == 0) {
+        const double2 rho_new = make_double2(acc[0], acc[1]);
+        const double rnew = sqrt(acc[2]);
+        double2 b = make_double2(0.0, 0.0);
+        int bad = MSB_OK, f = 0;
+        if (!cfinite(rho_new) || !isfinite(rnew)) {
+            bad = MSB_ENONFINITE;
+        } else if (rnew == 0.0) {
+            // exact solution: every shift converged
+        } else if (rho_new.x == 0.0 && rho_new.y == 0.0) {
+            bad = MSB_EBREAKDOWN;                           // (r, r) = 0 with r != 0
+        } else {
+            b = cdiv1(rho_new, st->rho);
             // bring ||r~|| back near ||b|| once it drifts by more than 2^20
-            const double ratio = rn / st->bnorm;
+            const double ratio = rnew / st->bnorm;
             if (ratio < 0x1p-20 || ratio > 0x1p20) f = -ilogb(ratio);
         }
-        st->rnorm = ldexp(rn, -st->sexp);
-        s_rn = rn;
-        s_rho = rho_new;
-        s_f = f;
-        s_m = st->m;
-    }
-    __syncthreads();
-    const double thr = st->tol * st->bnorm;
-    int still = 0;
-    for (int k = threadIdx.x; k < ns; k += blockDim.x) {
-        if (!sh.active[k]) continue;
-        // ||r^k_{m+1}|| = ||r~_{m+1}|| 2^{E_k} / |zeta~_{m+1}|
-        const double rk = ldexp(s_rn / cabs(sh.zeta[k]), sh.zexp[k]);
-        sh.iters[k] = s_m;
-        sh.resid[k] = rk / st->bnorm;
-        const double2 iz = cdiv(make_double2(1.0, 0.0), sh.zeta[k]);
-        sh.fz_coef[k] = make_double2(ldexp(iz.x, sh.zexp[k]), ldexp(iz.y, sh.zexp[k]));
-        sh.fz_iter[k] = s_m;
-        if (rk <= thr) { sh.active[k] = 0; sh.conv[k] = 1; }
-        else ++still;
-    }
-    double cnt[1] = {double(still)};
-    block_sum<1>(cnt, sm);
-    if (threadIdx.x == 0) {
-        st->nactive = int(cnt[0]);
-        if (s_stop || cnt[0] == 0.0 || s_m >= st->maxit) {
-            st->done = 1;
-            s_f = 0;                                   // nothing follows: keep r~ unscaled
-        }
-        const int f = s_f;
-        st->rho = make_double2(ldexp(s_rho.x, 2 * f), ldexp(s_rho.y, 2 * f));
-        st->fexp = f;
-        st->sexp += f;
-    }
-    __syncthreads();
-    if (s_f != 0) {
-        // S_{m+1} = S_m 2^f: exponents and residual factors of the shifts tested here
-        for (int k = threadIdx.x; k < ns; k += blockDim.x) {
-            if (sh.fz_iter[k] != s_m) continue;
-            sh.zexp[k] -= s_f;
-            const double2 c = sh.fz_coef[k];
-            sh.fz_coef[k] = make_double2(ldexp(c.x, -s_f), ldexp(c.y, -s_f));
-        }
+        st->beta_n = b;
+        st->rho_n = rho_new;
+        st->rn_n = rnew;
+        st->f_n = f;
+        st->bad_n = bad;
     }
 }
 
-// p = 2^f (r_{m+1} + beta p), r_{m+1} <- 2^f r_{m+1} (exact power-of-two rescale)
+// Convergence of every shift, iteration bookkeeping (one CTA).
+// fz_coef is the factor from the stored r~_{m+1} (rescaled by 2^f) to each tested
+// shift's recursive residual.
+__device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays& sh, int ns, int* s_still) {
+    const int m = st->m + 1, f = st->f_n, bad = st->bad_n;
+    const double rn = st->rn_n;
+    if (threadIdx.x == 0) *s_still = 0;
+    __syncthreads();
+    if (threadIdx.x < ns) {
+        const double thr = st->tol * st->bnorm, ib = st->ibnorm;
+        int still = 0;
+        for (int k = threadIdx.x; k < ns; k += blockDim.x) {
+            if (!sh.active[k]) continue;
+            // ||r^k_{m+1}|| = ||r~_{m+1}|| 2^{E_k} / |zeta~_{m+1}|
+            const int ze = sh.zexp[k];
+            const double2 iz = sh.izeta[k];
+            const double rk = scale2(rn * sqrt(fma(iz.x, iz.x, iz.y * iz.y)), ze);
+            sh.iters[k] = m;
+            sh.resid[k] = rk * ib;
+            sh.fz_coef[k] = scale2(iz, ze - f);
+            sh.fz_iter[k] = m;
+            sh.zexp[k] = ze - f;                           // S_{m+1} = S_m 2^f
+            if (rk <= thr) { sh.active[k] = 0; sh.conv[k] = 1; }
+            else ++still;
+        }
+        if (still) atomicAdd(s_still, still);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        st->m = m;
+        st->j = st->jcur + 1;
+        st->alpha_prev = st->alpha;
+        st->beta = st->beta_n;
+        st->rho = scale2(st->rho_n, 2 * f);
+        st->rnorm = scale2(rn, -st->sexp);
+        st->fexp = f;
+        st->sexp += f;
+        st->nactive = *s_still;
+        if (bad) st->status = bad;
+        if (bad || *s_still == 0 || m >= st->maxit) st->stop = 1;
+    }
+}
+
+// p = 2^f (r_{m+1} + beta p), r_{m+1} <- 2^f r_{m+1} (exact power-of-two rescale).
+// CTA 0: the per-shift convergence tests.
 // Dual form (rt != null): also p~ = 2^f (r~ + conj(beta) p~), r~ <- 2^f r~.
 template <typename V>
-__global__ void __launch_bounds__(256) k_update_p(V* ring, V* __restrict__ p, int64_t n,
-                                                  const SeedState* __restrict__ st, V* __restrict__ rt,
-                                                  V* __restrict__ pt) {
-    if (st->done) return;
-    V* __restrict__ r = ring + int64_t(st->slot) * n;
-    const double2 b = st->beta;
-    const int f = st->fexp;
-    if (f == 0) {
-        for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n;
-             s += int64_t(gridDim.x) * blockDim.x) {
-            p[s] = vadd(r[s], cscale(b.x, b.y, p[s]));
-            if (rt) pt[s] = vadd(rt[s], cscale(b.x, -b.y, pt[s]));
+__global__ void __launch_bounds__(kVecThreads) k_update_p(V* ring, int64_t ld, V* __restrict__ p, int64_t n, int nslot,
+                                                          SeedState* __restrict__ st, V* __restrict__ rt,
+                                                          V* __restrict__ pt, ShiftArrays sh, int ns) {
+    if (st->halted) return;
+    if (blockIdx.x == 0) {
+        __shared__ int s_still;
+        if (st->bad) {
+            if (threadIdx.x == 0) st->stop = 1;
+        } else {
+            shift_scalars_b(st, sh, ns, &s_still);
+        }
+        return;
+    }
+    if (st->bad || st->bad_n) return;
+    const double2 b = st->beta_n;
+    const int f = st->f_n;
+    V* __restrict__ r = ring + int64_t((st->slot0 + st->jcur + 1) % nslot) * ld;
+    const int64_t nth = int64_t(gridDim.x - 1) * blockDim.x, t0 = int64_t(blockIdx.x - 1) * blockDim.x + threadIdx.x;
+    const V bv = from_d2<V>(b);
+    if (f == 0 && !rt) {
+        if constexpr (std::is_same<V, float2>::value) {
+            const int64_t h = n >> 1;
+            const float4* __restrict__ r4 = reinterpret_cast<const float4*>(r);
+            float4* __restrict__ p4 = reinterpret_cast<float4*>(p);
+            auto one = [&](float4 x, float4 q) {
+                const float2 u = axpy_rn(make_float2(x.x, x.y), bv, make_float2(q.x, q.y), 1.f);
+                const float2 w = axpy_rn(make_float2(x.z, x.w), bv, make_float2(q.z, q.w), 1.f);
+                return make_float4(u.x, u.y, w.x, w.y);
+            };
+            int64_t i = t0;
+            for (; i + nth < h; i += 2 * nth) {
+                const float4 x0 = r4[i], q0 = p4[i], x1 = r4[i + nth], q1 = p4[i + nth];
+                p4[i] = one(x0, q0);
+                p4[i + nth] = one(x1, q1);
+            }
+            if (i < h) p4[i] = one(r4[i], p4[i]);
+            if ((n & 1) && t0 == 0) p[n - 1] = axpy_rn(r[n - 1], bv, p[n - 1], 1.f);
+        } else {
+            int64_t i = t0;
+            for (; i + nth < n; i += 2 * nth) {
+                const V x0 = r[i], q0 = p[i], x1 = r[i + nth], q1 = p[i + nth];
+                p[i] = cfma(bv, q0, x0);
+                p[i + nth] = cfma(bv, q1, x1);
+            }
+            if (i < n) p[i] = cfma(bv, p[i], r[i]);
         }
     } else {
         const double sc = ldexp(1.0, f);
-        for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n;
-             s += int64_t(gridDim.x) * blockDim.x) {
+        for (int64_t s = t0; s < n; s += nth) {
             const V rs = r[s];
             p[s] = cscale(sc, 0.0, vadd(rs, cscale(b.x, b.y, p[s])));
-            r[s] = cscale(sc, 0.0, rs);
+            if (f != 0) r[s] = cscale(sc, 0.0, rs);
             if (rt) {
                 const V ts = rt[s];
                 pt[s] = cscale(sc, 0.0, vadd(ts, cscale(b.x, -b.y, pt[s])));
-                rt[s] = cscale(sc, 0.0, ts);
+                if (f != 0) rt[s] = cscale(sc, 0.0, ts);
             }
         }
     }
 }
 
 // Start of a block of iterations: nothing pending for any shift.
-__global__ void k_block_begin(SeedState* st, ShiftArrays sh, int ns) {
+__global__ void k_block_begin(SeedState* st, ShiftArrays sh, int ns, int nslot) {
     for (int k = threadIdx.x; k < ns; k += blockDim.x) sh.nblk[k] = 0;
     if (threadIdx.x == 0) {
+        st->slot0 = (st->slot0 + st->j) % nslot;
         st->m0 = st->m;
         st->j = 0;
     }
@@ -413,7 +565,7 @@ __global__ void __launch_bounds__(256) k_flush(const V* __restrict__ ring, int n
     __shared__ int s_list[kMaxShifts];
     __shared__ int s_cnt;
     const int m0 = st->m0;
-    const int slot0 = ((st->slot - st->j) % nslot + nslot) % nslot;   // slot of r_{m0}
+    const int slot0 = st->slot0;                                      // slot of r_{m0}
     if (threadIdx.x == 0) {
         int c = 0;
         for (int k = 0; k < ns; ++k)
@@ -461,7 +613,7 @@ __global__ void __launch_bounds__(256) k_flush(const V* __restrict__ ring, int n
             }
             Pk[e] = pk;
             Xk[e] = xk;
-            if (rrec && (!sh.active[k] || st->done)) {
+            if (rrec && (!sh.active[k] || st->stop)) {
                 const int i = sh.fz_iter[k] - m0;                // 1 .. j
                 const V rf = ring[int64_t((slot0 + i) % nslot) * n_seed + src];
                 const double2 cf = sh.fz_coef[k];
@@ -530,12 +682,18 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         st->beta = make_double2(0.0, 0.0);
         st->rnorm = bn;
         st->bnorm = bn;
+        st->ibnorm = bn > 0.0 ? 1.0 / bn : 0.0;
         st->tol = tol;
-        st->m = 0; st->m0 = 0; st->j = 0; st->slot = 0;
+        st->m = 0; st->m0 = 0; st->j = 0; st->jcur = 0; st->slot0 = 0;
         st->status = MSB_OK;
         st->maxit = maxit;
-        st->done = (bn == 0.0 || maxit <= 0) ? 1 : 0;
-        if (bn != 0.0 && st->rho.x == 0.0 && st->rho.y == 0.0) { st->status = MSB_EBREAKDOWN; st->done = 1; }
+        st->halted = 0;
+        st->bad = 0;
+        st->bad_n = 0;
+        st->cnt_a = 0;
+        st->cnt_b = 0;
+        st->stop = (bn == 0.0 || maxit <= 0) ? 1 : 0;
+        if (bn != 0.0 && st->rho.x == 0.0 && st->rho.y == 0.0) { st->status = MSB_EBREAKDOWN; st->stop = 1; }
         st->nactive = bn == 0.0 ? 0 : ns;
         st->fexp = 0;
         st->sexp = 0;
@@ -546,6 +704,7 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         sh.shift[k] = shifts[k];
         sh.zeta[k] = make_double2(1.0, 0.0);
         sh.zeta_prev[k] = make_double2(1.0, 0.0);
+        sh.izeta[k] = make_double2(1.0, 0.0);
         sh.active[k] = s_bn == 0.0 ? 0 : 1;
         sh.conv[k] = s_bn == 0.0 ? 1 : 0;
         sh.broken[k] = 0;
@@ -573,14 +732,15 @@ struct SolverImpl {
     using C = V;
     const SolveProblem& pr;
     cudaStream_t st;
-    int nslot, B, grid_vec, grid_flush, grid_mvm;
+    int nslot, B, grid_vec, grid_flush, grid_mvm, grid_upd;
+    int64_t ld = 0;               // ring slot stride: n rounded up to even (16-byte FP32 pairs)
     RowPlan rows;                 // row-tiled seed product (Hubbard without a second amplitude or phases)
     const HubPart* rparts = nullptr;
     DevBuf<V> ring, p, v, Pbuf;
     DevBuf<V> rt, pt, vt;     // dual-space vectors (App. A), allocated only for the dual form
     DevBuf<double> part;
     DevBuf<SeedState> state;
-    DevBuf<double2> zeta, zeta_prev, shift, coef64;
+    DevBuf<double2> zeta, zeta_prev, izeta, shift, coef64;
     DevBuf<C> coefv;
     DevBuf<int> active, conv, broken, nblk, iters, zexp, fz_iter;
     DevBuf<double2> fz_coef;
@@ -602,13 +762,9 @@ struct SolverImpl {
             ProfScope ps("seed_mvm", st, 2 * nb + op->matrix_bytes(csz), op->hx_flops() + 16.0 * n);
             if (rows.ok)
                 launch_hub_rows<V>(rows, rparts, p.p, n, 1, pr.c0.x,
-                                   MvmEpi<V>{v.p, state.p, part.p, pt.p, pr.c0.y, {0.0, 0.0}, {}}, st);
+                                   MvmEpi<V>{v.p, state.p, part.p, pt.p, pr.c0.x, pr.c0.y, {0.0, 0.0}, {}}, st);
             else
                 k_mvm_dot<View, V><<<grid_vec, 256, 0, st>>>(view, p.p, v.p, n, pr.c0.x, pr.c0.y, state.p, part.p, pt.p);
-        }
-        {
-            ProfScope ps("shift_scalars", st, 0, 0);
-            k_scalar_a<C><<<1, kScalarThreads, 0, st>>>(state.p, part.p, grid_mvm, sh, pr.ns, B);
         }
         if (pr.dual) {
             ProfScope ps("seed_mvm", st, 2 * nb + op->matrix_bytes(csz), op->hx_flops() + 8.0 * n);
@@ -616,15 +772,13 @@ struct SolverImpl {
         }
         {
             ProfScope ps("seed_update", st, (pr.dual ? 6 : 3) * nb, 20.0 * n);
-            k_seed_update<V><<<grid_vec, 256, 0, st>>>(ring.p, v.p, n, nslot, state.p, part.p, rt.p, vt.p);
-        }
-        {
-            ProfScope ps("shift_scalars", st, 0, 0);
-            k_scalar_b<<<1, kScalarThreads, 0, st>>>(state.p, part.p, grid_vec, sh, pr.ns, nslot);
+            k_seed_update<V><<<grid_upd + 1, kVecThreads, 0, st>>>(ring.p, ld, v.p, n, nslot, state.p, part.p,
+                                                                   rt.p, vt.p, sh, pr.ns, B);
         }
         {
             ProfScope ps("seed_p", st, 3 * nb, 8.0 * n);
-            k_update_p<V><<<grid_vec, 256, 0, st>>>(ring.p, p.p, n, state.p, rt.p, pt.p);
+            k_update_p<V><<<grid_upd + 1, kVecThreads, 0, st>>>(ring.p, ld, p.p, n, nslot, state.p, rt.p,
+                                                                pt.p, sh, pr.ns);
         }
     }
 
@@ -633,7 +787,7 @@ struct SolverImpl {
         switch (B) {
 #define MSB_FLUSH_CASE(BB)                                                                          \
     case BB:                                                                                        \
-        k_flush<V, BB><<<grid_flush, 256, 0, st>>>(ring.p, nslot, pr.n, Pbuf.p, (V*)pr.x, pr.n_out, \
+        k_flush<V, BB><<<grid_flush, 256, 0, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, \
                                                    pr.rows, pr.rowlen, sh, pr.ns, state.p,          \
                                                    (V*)pr.rrec);                                    \
         break;
@@ -647,7 +801,7 @@ struct SolverImpl {
     void one_block_direct(const View& view) {
         {
             ProfScope ps("shift_scalars", st, 0, 0);
-            k_block_begin<<<1, kScalarThreads, 0, st>>>(state.p, sh, pr.ns);
+            k_block_begin<<<1, kScalarThreads, 0, st>>>(state.p, sh, pr.ns, nslot);
         }
         for (int i = 0; i < B; ++i) iteration(view);
         flush();
@@ -665,14 +819,16 @@ struct SolverImpl {
         rows = op->kind == 2 ? (f32 ? op->plan32 : op->plan64) : row_plan<V>(op, 1);
         if (op->kind == 2) rparts = f32 ? op->parts32.p : op->parts64.p;
         grid_mvm = rows.ok ? rows.grid : grid_vec;
-        ring.alloc(size_t(nslot) * n);
+        ld = (n + 1) / 2 * 2;
+        grid_upd = grid_for((n * int64_t(sizeof(V)) + 15) / 16, kVecThreads, 2);
+        ring.alloc(size_t(nslot) * ld);
         p.alloc(n);
         v.alloc(n);
         if (pr.dual) { rt.alloc(n); pt.alloc(n); vt.alloc(n); }
         Pbuf.alloc(size_t(ns) * pr.n_out);
-        part.alloc(size_t(std::max(grid_vec, grid_mvm)) * 4);
+        part.alloc(size_t(std::max(std::max(grid_vec, grid_mvm), grid_upd)) * 4);
         state.alloc(1);
-        zeta.alloc(ns); zeta_prev.alloc(ns); shift.alloc(ns);
+        zeta.alloc(ns); zeta_prev.alloc(ns); izeta.alloc(ns); shift.alloc(ns);
         coef64.alloc(size_t(ns) * B * 2);
         coefv.alloc(size_t(ns) * B * 2);
         active.alloc(ns); conv.alloc(ns); broken.alloc(ns); nblk.alloc(ns); iters.alloc(ns); zexp.alloc(ns);
@@ -680,7 +836,7 @@ struct SolverImpl {
         resid.alloc(ns);
         shifts_dev.alloc(ns);
         shifts_dev.upload(pr.shifts.data(), ns, st);
-        sh = ShiftArrays{zeta.p, zeta_prev.p, shift.p, coef64.p, (void*)coefv.p,
+        sh = ShiftArrays{zeta.p, zeta_prev.p, izeta.p, shift.p, coef64.p, (void*)coefv.p,
                          active.p, conv.p, broken.p, nblk.p, iters.p, resid.p, zexp.p, fz_coef.p, fz_iter.p};
 
         {
@@ -694,7 +850,7 @@ struct SolverImpl {
         }
         launches += 2;
         MSB_LAUNCH_CHECK();
-        const int64_t per_block = 2 + (pr.dual ? 6 : 5) * int64_t(B);   // kernels per block of iterations
+        const int64_t per_block = 2 + (pr.dual ? 4 : 3) * int64_t(B);   // kernels per block of iterations
         const int64_t max_blocks = (int64_t(pr.maxit) + B - 1) / B + 1;
         int64_t blocks = 0;
         if (prof_on()) {
@@ -710,7 +866,7 @@ struct SolverImpl {
                 const double no = double(pr.n_out) * csz;
                 prof_patch_last("shift_update", hs.flush_J * no + hs.flush_cnt * (hs.flush_first ? 2.0 : 4.0) * no,
                                 16.0 * hs.flush_cnt * hs.flush_J * double(pr.n_out));
-                if (hs.done || blocks > max_blocks + 2) break;
+                if (hs.stop || blocks > max_blocks + 2) break;
             }
             prof_collect();
             out.flushes = blocks;
@@ -720,7 +876,7 @@ struct SolverImpl {
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
         MSB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        k_block_begin<<<1, kScalarThreads, 0, st>>>(state.p, sh, int(ns));
+        k_block_begin<<<1, kScalarThreads, 0, st>>>(state.p, sh, int(ns), nslot);
         for (int i = 0; i < B; ++i) iteration(view);
         flush();
         MSB_CUDA(cudaStreamEndCapture(st, &graph));
@@ -741,7 +897,7 @@ struct SolverImpl {
             MSB_CUDA(cudaEventRecord(ev[slot], st));
             if (blocks >= 1) {
                 MSB_CUDA(cudaEventSynchronize(ev[slot ^ 1]));
-                if (hstate.p[slot ^ 1].done) finished = true;
+                if (hstate.p[slot ^ 1].stop) finished = true;
             }
             ++blocks;
             if (blocks > max_blocks + 2) break;

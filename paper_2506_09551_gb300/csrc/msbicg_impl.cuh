@@ -13,6 +13,7 @@ constexpr int kMaxShifts = 4096;
 struct ShiftArrays {
     double2* zeta;        // zeta^k_m
     double2* zeta_prev;   // zeta^k_{m-1}
+    double2* izeta;       // 1 / zeta^k_m
     double2* shift;       // s_k
     double2* coef64;      // [k][B][2]: (gamma, c) of each iteration of the block, FP64
     void* coefv;          // same in the vector precision (double2 or float2)

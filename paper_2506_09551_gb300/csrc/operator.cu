@@ -224,16 +224,16 @@ template <typename V>
 struct ApplyEpi {
     V* y;
     int64_t n;
-    double c0i;
+    double c0r, c0i;
     __device__ __forceinline__ bool stop() const { return false; }
     __device__ __forceinline__ void begin(int col) { y += int64_t(col) * n; }
     template <typename S>
-    __device__ __forceinline__ void operator()(int64_t s, V xs, V acc, S dg, S mt) {
-        y[s] = hub_value(acc, dg, mt, S(c0i), xs);
+    __device__ __forceinline__ void operator()(int64_t s, V xs, V acc, S dg, S mt, S shift) {
+        y[s] = hub_value(acc, dg, mt, shift, c0r, c0i, xs);
     }
     __device__ __forceinline__ void pair(int64_t s, float2 xa, float2 xb, float2 a, float2 b, float da, float db,
-                                         float mt) {
-        const float2 p = hub_value(a, da, mt, float(c0i), xa), q = hub_value(b, db, mt, float(c0i), xb);
+                                         float mt, float shift) {
+        const float2 p = hub_value(a, da, mt, shift, c0r, c0i, xa), q = hub_value(b, db, mt, shift, c0r, c0i, xb);
         *reinterpret_cast<float4*>(y + s) = make_float4(p.x, p.y, q.x, q.y);
     }
     __device__ __forceinline__ void finish(double*) const {}
@@ -249,7 +249,7 @@ static bool launch_apply_rows(const msb_op* op, double2 c0, const void* x, void*
     const int64_t n = op->dim;
     ProfScope ps("h_apply", st, nvec * 2.0 * n * sizeof(V), nvec * (op->hx_flops() + 8.0 * n));
     launch_hub_rows<V>(p, op->kind == 2 ? (f32 ? op->parts32.p : op->parts64.p) : nullptr, (const V*)x, n, nvec, c0.x,
-                       ApplyEpi<V>{(V*)y, n, c0.y}, st);
+                       ApplyEpi<V>{(V*)y, n, c0.x, c0.y}, st);
     MSB_LAUNCH_CHECK();
     count_launch();
     return true;
