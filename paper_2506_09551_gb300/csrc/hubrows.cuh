@@ -266,7 +266,7 @@ RowPlan row_plan(const msb_op* op, int nvec) {
         q.split = 1;
         // halve the rows' work while a column has fewer than ~12 tiles per SM and a part
         // still has two elements per thread
-        while (q.R == 1 && q.split < 4 && q.v.Dup * q.split * ops.size() * nvec < int64_t(sm_count()) * 12 &&
+        while (q.R == 1 && q.split < 4 && q.v.Dup * q.split * int64_t(ops.size()) * nvec < int64_t(sm_count()) * 12 &&
                q.v.Ddn / (2 * q.split) >= 2 * p.threads * pe)
             q.split *= 2;
         const size_t sm = size_t(q.R) * (q.v.Ddn + 2) * sizeof(V) + (3 * (q.v.L + 1) + q.R * q.v.Wup) * sizeof(scalar_t<V>) +

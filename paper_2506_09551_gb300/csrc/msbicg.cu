@@ -41,6 +41,7 @@
 #include <cmath>
 #include <memory>
 
+#include "flush_tc.cuh"
 #include "hubrows.cuh"
 #include "kernels.cuh"
 #include "msbicg_impl.cuh"
@@ -81,6 +82,7 @@ struct SeedState {
     int fexp;             // r~_m, p~_m were rescaled by 2^fexp after r_m was formed
     int sexp;             // log2 S_m (for reporting the true seed residual)
     int flush_J, flush_cnt, flush_first;   // work of the last fused update (profiling)
+    int rexp[kTcWindow + 1];               // per ring slot: exponent of the stored ||r~||
 };
 
 // ---------------------------------------------------------------------------
@@ -433,7 +435,7 @@ __global__ void __launch_bounds__(kVecThreads) k_seed_update(V* ring, int64_t ld
 // Convergence of every shift, iteration bookkeeping (one CTA).
 // fz_coef is the factor from the stored r~_{m+1} (rescaled by 2^f) to each tested
 // shift's recursive residual.
-__device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays& sh, int ns, int* s_still) {
+__device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays& sh, int ns, int nslot, int* s_still) {
     const int m = st->m + 1, f = st->f_n, bad = st->bad_n;
     const double rn = st->rn_n;
     if (threadIdx.x == 0) *s_still = 0;
@@ -461,6 +463,7 @@ __device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays
     if (threadIdx.x == 0) {
         st->m = m;
         st->j = st->jcur + 1;
+        st->rexp[(st->slot0 + st->jcur + 1) % nslot] = rn > 0.0 && isfinite(rn) ? ilogb(rn) + f : 0;
         st->alpha_prev = st->alpha;
         st->beta = st->beta_n;
         st->rho = scale2(st->rho_n, 2 * f);
@@ -486,7 +489,7 @@ __global__ void __launch_bounds__(kVecThreads) k_update_p(V* ring, int64_t ld, V
         if (st->bad) {
             if (threadIdx.x == 0) st->stop = 1;
         } else {
-            shift_scalars_b(st, sh, ns, &s_still);
+            shift_scalars_b(st, sh, ns, nslot, &s_still);
         }
         return;
     }
@@ -548,39 +551,37 @@ __global__ void k_block_begin(SeedState* st, ShiftArrays sh, int ns, int nslot) 
     }
 }
 
-// Lagged fused per-shift update over the block's iterations (Eqs. 7-8):
+// Lagged fused per-shift update over the window's iterations (Eqs. 7-8):
 // for every shift with pending iterations, P <- r_i + gamma_i P; x <- x + c_i P
-// for i = 0 .. nblk[k]-1, P and x held in registers, r_i from the ring.
+// for i = 0 .. nblk[k]-1, r_i from the ring, BMAX iterations at a time with P and x in
+// registers.  The order of the operations does not depend on the window.
 // Optional row map: element e of the per-shift vectors is seed element
 // rows[e / rowlen] * rowlen + e % rowlen (only the rows the caller needs).
-// rrec (optional): for a shift that froze in this block, or for every shift with
-// pending iterations once the solve is done, its recursive residual at its last
-// tested iteration, fz_coef[k] * r~_{fz_iter[k]} (r~ from the ring).
+// FP32 (BMAX = 32, the whole window in one pass): with 16 FMAs per 8 bytes of r and 256
+// per 32 bytes of P and x, the FP32 pipe and DRAM are about balanced; the next shift's P
+// and x are loaded before the current one's arithmetic.  Measured (48 shifts, n = 2.9 M,
+// against a window of 8): see the FP32 solve in the commit that brought it.
+// FP64: bound by the FP64 pipe (8 FMAs per shift, element and iteration); windows with many
+// shifts go to the tensor cores (flush_tc.cuh), and this kernel returns at once.
 template <typename V, int BMAX>
-__global__ void __launch_bounds__(256) k_flush(const V* __restrict__ ring, int nslot, int64_t n_seed,
-                                               V* __restrict__ P, V* __restrict__ X, int64_t n_out,
-                                               const int32_t* __restrict__ rows, int64_t rowlen,
-                                               ShiftArrays sh, int ns, SeedState* __restrict__ st,
-                                               V* __restrict__ rrec) {
+__global__ void __launch_bounds__(256, 2) k_flush(const V* __restrict__ ring, int nslot, int64_t ld,
+                                                  V* __restrict__ P, V* __restrict__ X, int64_t n_out,
+                                                  const int32_t* __restrict__ rows, int64_t rowlen,
+                                                  ShiftArrays sh, int ns, SeedState* __restrict__ st, int W,
+                                                  const int* __restrict__ tc_cnt) {
     __shared__ int s_list[kMaxShifts];
     __shared__ int s_cnt;
-    const int m0 = st->m0;
-    const int slot0 = st->slot0;                                      // slot of r_{m0}
-    if (threadIdx.x == 0) {
-        int c = 0;
-        for (int k = 0; k < ns; ++k)
-            if (sh.nblk[k] > 0) s_list[c++] = k;
-        s_cnt = c;
-        if (blockIdx.x == 0) {
-            st->flush_J = st->j;
-            st->flush_cnt = c;
-            st->flush_first = m0 == 0;
-        }
+    const bool tc = tc_cnt != nullptr && tc_use(*tc_cnt, st->bnorm);
+    if (tc && blockIdx.x != 0) return;
+    const int cnt = pending_list(sh.nblk, ns, 0, s_list, &s_cnt);
+    const bool first = st->m0 == 0;
+    const int slot0 = st->slot0, JW = st->j;                          // slot of r_{m0}
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->flush_J = JW;
+        st->flush_cnt = cnt;
+        st->flush_first = first;
     }
-    __syncthreads();
-    const int cnt = s_cnt;
-    if (cnt == 0) return;
-    const bool first = (m0 == 0);
+    if (tc || cnt == 0) return;
     const V* __restrict__ coef = reinterpret_cast<const V*>(sh.coefv);
     for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < n_out;
          e += int64_t(gridDim.x) * blockDim.x) {
@@ -589,37 +590,71 @@ __global__ void __launch_bounds__(256) k_flush(const V* __restrict__ ring, int n
             const int64_t row = e / rowlen;
             src = int64_t(__ldg(rows + row)) * rowlen + (e - row * rowlen);
         }
-        V r[BMAX];
-#pragma unroll
-        for (int i = 0; i < BMAX; ++i) {
-            const int sl = (slot0 + i) % nslot;
-            r[i] = (i < st->j) ? ring[int64_t(sl) * n_seed + src] : vzero(V{});
-        }
-        for (int q = 0; q < cnt; ++q) {
-            const int k = s_list[q];
-            const int J = sh.nblk[k];
-            V* __restrict__ Pk = P + int64_t(k) * n_out;
-            V* __restrict__ Xk = X + int64_t(k) * n_out;
-            V pk = first ? vzero(V{}) : Pk[e];
-            V xk = first ? vzero(V{}) : Xk[e];
-            const V* ck = coef + int64_t(k) * BMAX * 2;
+        for (int i0 = 0; i0 < JW; i0 += BMAX) {
+            const bool fresh = first && i0 == 0;
+            V r[BMAX];
 #pragma unroll
             for (int i = 0; i < BMAX; ++i) {
-                if (i < J) {
-                    const V g = ck[2 * i], c = ck[2 * i + 1];
-                    pk = cfma(g, pk, r[i]);    // P = r_i + gamma_i P
-                    xk = cfma(c, pk, xk);      // x = x + c_i P
-                }
+                const int sl = (slot0 + i0 + i) % nslot;
+                r[i] = (i0 + i < JW) ? ring[int64_t(sl) * ld + src] : vzero(V{});
             }
-            Pk[e] = pk;
-            Xk[e] = xk;
-            if (rrec && (!sh.active[k] || st->stop)) {
-                const int i = sh.fz_iter[k] - m0;                // 1 .. j
-                const V rf = ring[int64_t((slot0 + i) % nslot) * n_seed + src];
-                const double2 cf = sh.fz_coef[k];
-                rrec[int64_t(k) * n_out + e] = cscale(cf.x, cf.y, rf);
+            int k = s_list[0];
+            V np = fresh ? vzero(V{}) : P[int64_t(k) * n_out + e];
+            V nx = fresh ? vzero(V{}) : X[int64_t(k) * n_out + e];
+            for (int q = 0; q < cnt; ++q) {
+                const int kc = k;
+                V pk = np, xk = nx;
+                if (q + 1 < cnt) {
+                    k = s_list[q + 1];
+                    if (!fresh) {
+                        np = P[int64_t(k) * n_out + e];
+                        nx = X[int64_t(k) * n_out + e];
+                    }
+                }
+                const int J = sh.nblk[kc] - i0;
+                if (J <= 0) continue;
+                const V* __restrict__ ck = coef + (int64_t(kc) * W + i0) * 2;
+                if (J >= BMAX) {
+#pragma unroll
+                    for (int i = 0; i < BMAX; ++i) {
+                        pk = cfma(ck[2 * i], pk, r[i]);        // P = r_i + gamma_i P
+                        xk = cfma(ck[2 * i + 1], pk, xk);      // x = x + c_i P
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < BMAX; ++i) {
+                        if (i >= J) break;
+                        pk = cfma(ck[2 * i], pk, r[i]);
+                        xk = cfma(ck[2 * i + 1], pk, xk);
+                    }
+                }
+                P[int64_t(kc) * n_out + e] = pk;
+                X[int64_t(kc) * n_out + e] = xk;
             }
         }
+    }
+}
+
+// For a shift that froze in this window, or for every shift with pending iterations
+// once the solve is done, its recursive residual at its last tested iteration,
+// fz_coef[k] * r~_{fz_iter[k]} (r~ from the ring).  blockIdx.y: shift.
+template <typename V>
+__global__ void __launch_bounds__(256) k_rrec(const V* __restrict__ ring, int nslot, int64_t ld, V* __restrict__ rrec,
+                                              int64_t n_out, const int32_t* __restrict__ rows, int64_t rowlen,
+                                              ShiftArrays sh, const SeedState* __restrict__ st) {
+    const int k = blockIdx.y;
+    if (sh.nblk[k] == 0 || (sh.active[k] && !st->stop)) return;
+    const int i = sh.fz_iter[k] - st->m0;                             // 1 .. j
+    const V* __restrict__ r = ring + int64_t((st->slot0 + i) % nslot) * ld;
+    const double2 cf = sh.fz_coef[k];
+    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < n_out;
+         e += int64_t(gridDim.x) * blockDim.x) {
+        int64_t src = e;
+        if (rows) {
+            const int64_t row = e / rowlen;
+            src = int64_t(__ldg(rows + row)) * rowlen + (e - row * rowlen);
+        }
+        rrec[int64_t(k) * n_out + e] = cscale(cf.x, cf.y, r[src]);
     }
 }
 
@@ -683,6 +718,7 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         st->rnorm = bn;
         st->bnorm = bn;
         st->ibnorm = bn > 0.0 ? 1.0 / bn : 0.0;
+        st->rexp[0] = bn > 0.0 && isfinite(bn) ? ilogb(bn) : 0;
         st->tol = tol;
         st->m = 0; st->m0 = 0; st->j = 0; st->jcur = 0; st->slot0 = 0;
         st->status = MSB_OK;
@@ -733,6 +769,15 @@ struct SolverImpl {
     const SolveProblem& pr;
     cudaStream_t st;
     int nslot, B, grid_vec, grid_flush, grid_mvm, grid_upd;
+    // Window of the per-shift update: 32 iterations in FP32, 64 in FP64 (one contraction on
+    // the tensor cores), whatever the block B of iterations per graph; B when the ring of
+    // residuals would take too much memory.
+    int W = 0, grid_tc = 0;
+    bool tc = false;
+    TcCoef tcc{};
+    DevBuf<int> tc_list, tc_cnt, tc_exp;
+    DevBuf<double2> tc_mul;
+    DevBuf<uint4> tc_frag;
     int64_t ld = 0;               // ring slot stride: n rounded up to even (16-byte FP32 pairs)
     RowPlan rows;                 // row-tiled seed product (Hubbard without a second amplitude or phases)
     const HubPart* rparts = nullptr;
@@ -773,7 +818,7 @@ struct SolverImpl {
         {
             ProfScope ps("seed_update", st, (pr.dual ? 6 : 3) * nb, 20.0 * n);
             k_seed_update<V><<<grid_upd + 1, kVecThreads, 0, st>>>(ring.p, ld, v.p, n, nslot, state.p, part.p,
-                                                                   rt.p, vt.p, sh, pr.ns, B);
+                                                                   rt.p, vt.p, sh, pr.ns, W);
         }
         {
             ProfScope ps("seed_p", st, 3 * nb, 8.0 * n);
@@ -782,29 +827,35 @@ struct SolverImpl {
         }
     }
 
+    // End of a window: the per-shift update of its iterations, then an empty window.
     void flush() {
-        ProfScope ps("shift_update", st, 0, 0);
-        switch (B) {
-#define MSB_FLUSH_CASE(BB)                                                                          \
-    case BB:                                                                                        \
-        k_flush<V, BB><<<grid_flush, 256, 0, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, \
-                                                   pr.rows, pr.rowlen, sh, pr.ns, state.p,          \
-                                                   (V*)pr.rrec);                                    \
-        break;
-            MSB_FLUSH_CASE(1) MSB_FLUSH_CASE(2) MSB_FLUSH_CASE(4) MSB_FLUSH_CASE(8) MSB_FLUSH_CASE(16)
-#undef MSB_FLUSH_CASE
-            default: fail(MSB_EINVAL, "block must be 1, 2, 4, 8 or 16");
+        {
+            ProfScope ps("shift_update", st, 0, 0);
+            const int* cnt = tc ? tcc.cnt : nullptr;
+            if (tc) {
+                k_tc_coef<<<(pr.ns + 3) / 4, 128, 0, st>>>(nblk.p, coef64.p, pr.ns, W, nslot, &state.p->slot0,
+                                                          &state.p->bnorm, tcc);
+            }
+            constexpr int BMAX = std::is_same<V, float2>::value ? 32 : 8;
+            k_flush<V, BMAX><<<grid_flush, 256, 0, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, pr.rows, pr.rowlen,
+                                                         sh, pr.ns, state.p, W, cnt);
+            if constexpr (std::is_same<V, double2>::value) {
+                if (tc)
+                    k_flush_tc<<<grid_tc, kTcThreads, kTcSmem, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, pr.rows,
+                                                                     pr.rowlen, &state.p->slot0, &state.p->j,
+                                                                     &state.p->m0, &state.p->bnorm, tcc);
+            }
+            if (pr.rrec)
+                k_rrec<V><<<dim3(grid_for(pr.n_out, 256, 2), pr.ns), 256, 0, st>>>(ring.p, nslot, ld, (V*)pr.rrec, pr.n_out,
+                                                                                  pr.rows, pr.rowlen, sh, state.p);
         }
+        launches += 1 + (tc ? 2 : 0) + (pr.rrec ? 1 : 0);
     }
 
-    template <class View>
-    void one_block_direct(const View& view) {
-        {
-            ProfScope ps("shift_scalars", st, 0, 0);
-            k_block_begin<<<1, kScalarThreads, 0, st>>>(state.p, sh, pr.ns, nslot);
-        }
-        for (int i = 0; i < B; ++i) iteration(view);
-        flush();
+    void window_begin() {
+        ProfScope ps("shift_scalars", st, 0, 0);
+        k_block_begin<<<1, kScalarThreads, 0, st>>>(state.p, sh, pr.ns, nslot);
+        ++launches;
     }
 
     template <class View>
@@ -812,7 +863,7 @@ struct SolverImpl {
         op = op_;
         const int64_t n = pr.n, ns = pr.ns;
         B = pr.block;
-        nslot = B + 1;
+        W = std::is_same<V, float2>::value ? 32 : kTcWindow;
         grid_vec = grid_for(n, 256, 8);
         grid_flush = grid_for(pr.n_out, 256, 8);
         constexpr bool f32 = std::is_same<V, float2>::value;
@@ -821,7 +872,16 @@ struct SolverImpl {
         grid_mvm = rows.ok ? rows.grid : grid_vec;
         ld = (n + 1) / 2 * 2;
         grid_upd = grid_for((n * int64_t(sizeof(V)) + 15) / 16, kVecThreads, 2);
-        ring.alloc(size_t(nslot) * ld);
+        if (size_t(W + 1) * ld * sizeof(V) > (size_t(16) << 30)) W = B;
+        try {
+            ring.alloc(size_t(W + 1) * ld);
+        } catch (const Error& e) {
+            if (e.status != MSB_ENOMEM || W == B) throw;
+            cudaGetLastError();
+            W = B;
+            ring.alloc(size_t(W + 1) * ld);
+        }
+        nslot = W + 1;
         p.alloc(n);
         v.alloc(n);
         if (pr.dual) { rt.alloc(n); pt.alloc(n); vt.alloc(n); }
@@ -829,11 +889,19 @@ struct SolverImpl {
         part.alloc(size_t(std::max(std::max(grid_vec, grid_mvm), grid_upd)) * 4);
         state.alloc(1);
         zeta.alloc(ns); zeta_prev.alloc(ns); izeta.alloc(ns); shift.alloc(ns);
-        coef64.alloc(size_t(ns) * B * 2);
-        coefv.alloc(size_t(ns) * B * 2);
+        coef64.alloc(size_t(ns) * W * 2);
+        coefv.alloc(size_t(ns) * W * 2);
         active.alloc(ns); conv.alloc(ns); broken.alloc(ns); nblk.alloc(ns); iters.alloc(ns); zexp.alloc(ns);
         fz_iter.alloc(ns); fz_coef.alloc(ns);
         resid.alloc(ns);
+        tc = std::is_same<V, double2>::value && W == kTcWindow && ns >= kTcMinShifts;
+        if (tc) {
+            tc_list.alloc(ns); tc_cnt.alloc(1); tc_exp.alloc(2 * ns); tc_mul.alloc(2 * ns);
+            tc_frag.alloc(size_t((ns + 3) / 4) * kTcSteps * kTcDigits * 32);
+            tcc = TcCoef{tc_list.p, tc_cnt.p, tc_mul.p, tc_exp.p, tc_frag.p, state.p->rexp};
+            grid_tc = int(std::min<int64_t>((pr.n_out + kTcCols - 1) / kTcCols, 2 * sm_count()));
+            MSB_CUDA(cudaFuncSetAttribute((const void*)k_flush_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmem)));
+        }
         shifts_dev.alloc(ns);
         shifts_dev.upload(pr.shifts.data(), ns, st);
         sh = ShiftArrays{zeta.p, zeta_prev.p, izeta.p, shift.p, coef64.p, (void*)coefv.p,
@@ -850,35 +918,42 @@ struct SolverImpl {
         }
         launches += 2;
         MSB_LAUNCH_CHECK();
-        const int64_t per_block = 2 + (pr.dual ? 4 : 3) * int64_t(B);   // kernels per block of iterations
+        const int64_t per_block = (pr.dual ? 4 : 3) * int64_t(B);       // kernels per block of iterations
         const int64_t max_blocks = (int64_t(pr.maxit) + B - 1) / B + 1;
         int64_t blocks = 0;
         if (prof_on()) {
-            // Profiled: direct launches, one sync per block to attribute the
-            // fused update's work (shifts and iterations it carried).
+            // Profiled: direct launches, one sync per block, and one after each fused
+            // update to attribute its work (shifts and iterations it carried).
             SeedState hs;
-            for (;;) {
-                one_block_direct(view);
-                launches += per_block;
-                ++blocks;
+            auto look = [&] {
                 MSB_CUDA(cudaMemcpyAsync(&hs, state.p, sizeof(SeedState), cudaMemcpyDeviceToHost, st));
                 MSB_CUDA(cudaStreamSynchronize(st));
-                const double no = double(pr.n_out) * csz;
-                prof_patch_last("shift_update", hs.flush_J * no + hs.flush_cnt * (hs.flush_first ? 2.0 : 4.0) * no,
-                                16.0 * hs.flush_cnt * hs.flush_J * double(pr.n_out));
-                if (hs.stop || blocks > max_blocks + 2) break;
+            };
+            for (;;) {
+                for (int i = 0; i < B; ++i) iteration(view);
+                launches += per_block;
+                ++blocks;
+                look();
+                const bool end = hs.stop || blocks > max_blocks + 2;
+                if (end || blocks * B % W == 0) {
+                    flush();
+                    look();
+                    const double no = double(pr.n_out) * csz;
+                    prof_patch_last("shift_update", hs.flush_J * no + hs.flush_cnt * (hs.flush_first ? 2.0 : 4.0) * no,
+                                    16.0 * hs.flush_cnt * hs.flush_J * double(pr.n_out));
+                    window_begin();
+                }
+                if (end) break;
             }
             prof_collect();
             out.flushes = blocks;
         } else {
 
-        // One block of B iterations + the fused per-shift update, captured once.
+        // One block of B iterations, captured once.
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
         MSB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        k_block_begin<<<1, kScalarThreads, 0, st>>>(state.p, sh, int(ns), nslot);
         for (int i = 0; i < B; ++i) iteration(view);
-        flush();
         MSB_CUDA(cudaStreamEndCapture(st, &graph));
         MSB_CUDA(cudaGraphInstantiate(&exec, graph, 0));
 
@@ -892,6 +967,7 @@ struct SolverImpl {
         while (!finished) {
             MSB_CUDA(cudaGraphLaunch(exec, st));
             launches += per_block;
+            if ((blocks + 1) * B % W == 0) { flush(); window_begin(); }
             const int slot = int(blocks & 1);
             MSB_CUDA(cudaMemcpyAsync(&hstate.p[slot], state.p, sizeof(SeedState), cudaMemcpyDeviceToHost, st));
             MSB_CUDA(cudaEventRecord(ev[slot], st));
@@ -902,6 +978,8 @@ struct SolverImpl {
             ++blocks;
             if (blocks > max_blocks + 2) break;
         }
+        flush();                                       // the last, partial window (nothing pending: no work)
+        MSB_LAUNCH_CHECK();
         MSB_CUDA(cudaStreamSynchronize(st));
         cudaEventDestroy(ev[0]);
         cudaEventDestroy(ev[1]);
