@@ -264,20 +264,28 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_flush_tc(const double2* __res
         const int tkey = s_key;
         const bool tbad = tkey == INT_MAX;
         const int te = tkey == INT_MIN || tbad ? 0 : tc_exponent(tkey);
-        for (int i = ig; i < steps * 8; i += kTcThreads / kTcCols) {
-            unsigned long long ur = 0x0080808080808080ull, ui = ur;
-            if (src >= 0 && i < J && !tbad) {
-                const double2 r = ring[int64_t(s_slot[i]) * ld + src];
-                const int e = te + s_e[i];
-                ur = tc_fixed(r.x, e);
-                ui = tc_fixed(r.y, e);
+        // digits: a warp takes eight columns and one depth step; lane: column lane % 8,
+        // iterations lane / 8 and 4 more (whole 128-byte lines of r, conflict-free stores)
+        for (int c = wid; c < steps * (kTcCols / 8); c += kTcThreads / 32) {
+            const int s = c / (kTcCols / 8), nt = c % (kTcCols / 8), cl = lane & 7, ii = lane >> 3;
+            const int sc = s_src[nt * 8 + cl];
+            unsigned long long u[2][2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = s * 8 + ii + 4 * h;
+                u[h][0] = u[h][1] = 0x0080808080808080ull;
+                if (sc >= 0 && i < J && !tbad) {
+                    const double2 r = ring[int64_t(s_slot[i]) * ld + sc];
+                    const int e = te + s_e[i];
+                    u[h][0] = tc_fixed(r.x, e);
+                    u[h][1] = tc_fixed(r.y, e);
+                }
             }
-            const int s = i >> 3, ii = i & 7;
-            unsigned* __restrict__ b = reinterpret_cast<unsigned*>(s_b) +
-                                       (((s * (kTcCols / 8) + (col >> 3)) * 32 + (col & 7) * 4 + (ii & 3)) * 2 + (ii >> 2));
+            uint2* __restrict__ b = s_b + (s * (kTcCols / 8) + nt) * 32 + cl * 4 + ii;
 #pragma unroll
             for (int d = 0; d < kTcDigits; ++d)
-                b[d * (kTcSteps * (kTcCols / 8) * 64)] = tc_pack(tc_digit(ur, d), tc_digit(ui, d));
+                b[d * (kTcSteps * (kTcCols / 8) * 32)] = make_uint2(tc_pack(tc_digit(u[0][0], d), tc_digit(u[0][1], d)),
+                                                                   tc_pack(tc_digit(u[1][0], d), tc_digit(u[1][1], d)));
         }
         __syncthreads();
         const int nt0 = (wid & 3) * 2;

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
         }
         __syncthreads();
         const int core = h.core;
-        const S mt = S(-h.t);
+        const S mt = S(-h.t), shift = S(P.shift);
         const S s1 = S(one);                                       // 1, opaque to the compiler: an FMA, not an add
         const uint16_t* __restrict__ t16 = h.hdnr16;
         constexpr int PE = PAIR ? 2 : 1;
@@ -154,7 +154,15 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
                     hop_add(a, us[k], v0); hop_add(a, us[k + 1], v1);
                     hop_add(a, us[k + 2], v2); hop_add(a, us[k + 3], v3);
                 }
-                for (; k < nu; ++k) hop_add(a, us[k], x4[(uo[k] >> 1) + dh]);
+                if (k + 3 == nu) {
+                    const float4 v0 = x4[(uo[k] >> 1) + dh], v1 = x4[(uo[k + 1] >> 1) + dh], v2 = x4[(uo[k + 2] >> 1) + dh];
+                    hop_add(a, us[k], v0); hop_add(a, us[k + 1], v1); hop_add(a, us[k + 2], v2);
+                } else if (k + 2 == nu) {
+                    const float4 v0 = x4[(uo[k] >> 1) + dh], v1 = x4[(uo[k + 1] >> 1) + dh];
+                    hop_add(a, us[k], v0); hop_add(a, us[k + 1], v1);
+                } else if (k < nu) {
+                    hop_add(a, us[k], x4[(uo[k] >> 1) + dh]);
+                }
                 const uint32_t nn = __ldg(reinterpret_cast<const uint16_t*>(h.ndn) + dh);
                 const int nd = __reduce_max_sync(0xffffffffu, act ? max(nn & 0xFFu, nn >> 8) : 0u);
                 const uint32_t* __restrict__ tp = reinterpret_cast<const uint32_t*>(t16) + dh;
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
                 const float da = lut[__popc(su & sa) + na * (L + 1)], db = lut[__popc(su & sb) + nb * (L + 1)];
                 if (act) {
                     const float2 xa = xr[d], xb = xr[d + 1];
-                    epi.pair(base + e, xa, xb, make_float2(a.x, a.y), make_float2(a.z, a.w), da, db, mt, float(P.shift));
+                    epi.pair(base + e, xa, xb, make_float2(a.x, a.y), make_float2(a.z, a.w), da, db, mt, shift);
                 }
             } else {
                 V a = vzero(V{});
@@ -196,7 +204,16 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
                     hop_add(a, us[k], v0); hop_add(a, us[k + 1], v1);
                     hop_add(a, us[k + 2], v2); hop_add(a, us[k + 3], v3);
                 }
-                for (; k < nu; ++k) hop_add(a, us[k], xp[uo[k] + d]);
+                // the rest together, without FP64 work for missing hops
+                if (k + 3 == nu) {
+                    const V v0 = xp[uo[k] + d], v1 = xp[uo[k + 1] + d], v2 = xp[uo[k + 2] + d];
+                    hop_add(a, us[k], v0); hop_add(a, us[k + 1], v1); hop_add(a, us[k + 2], v2);
+                } else if (k + 2 == nu) {
+                    const V v0 = xp[uo[k] + d], v1 = xp[uo[k + 1] + d];
+                    hop_add(a, us[k], v0); hop_add(a, us[k + 1], v1);
+                } else if (k < nu) {
+                    hop_add(a, us[k], xp[uo[k] + d]);
+                }
                 const int nd = __reduce_max_sync(0xffffffffu, act ? unsigned(__ldg(h.ndn + d)) : 0u);
                 const uint16_t* __restrict__ tp = t16 + d;
                 k = 0;
@@ -213,7 +230,7 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
                 const uint32_t sd = __ldg(h.sdn + d);
                 const int nb = core >= 0 ? int((su >> core) & 1u) + int((sd >> core) & 1u) : 0;
                 const S dg = lut[__popc(su & sd) + nb * (L + 1)];
-                if (act) epi(base + e, xr[d], a, dg, mt, S(P.shift));
+                if (act) epi(base + e, xr[d], a, dg, mt, shift);
             }
         }
         __syncthreads();                                           // the tile's shared memory is reused
@@ -226,11 +243,10 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
 __device__ __forceinline__ double2 hub_value(double2 acc, double dg, double mt, double, double, double c0i, double2 x) {
     return make_double2(fma(mt, acc.x, fma(dg, x.x, -c0i * x.y)), fma(mt, acc.y, fma(dg, x.y, c0i * x.x)));
 }
-__device__ __forceinline__ float2 hub_value(float2 acc, float dg, float mt, float shift, double c0r, double c0i,
-                                            float2 x) {
+__device__ __forceinline__ float2 hub_value(float2 acc, float dg, float mt, float shift, float c0r, float c0i, float2 x) {
     float2 h = make_float2(__fmaf_rn(mt, acc.x, __fmul_rn(dg, x.x)), __fmaf_rn(mt, acc.y, __fmul_rn(dg, x.y)));
     if (shift != 0.f) h = vaxpy(shift, x, h);
-    const float2 c = cscale_rn(float(c0r), float(c0i), x);
+    const float2 c = cscale_rn(c0r, c0i, x);
     return make_float2(__fadd_rn(h.x, c.x), __fadd_rn(h.y, c.y));
 }
 

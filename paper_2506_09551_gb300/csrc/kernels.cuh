@@ -190,6 +190,17 @@ __device__ __forceinline__ void sum_partials_cg(const double* part, int n, doubl
     block_sum_sm<NV>(v, sm);
 }
 
+// a / b with one division: b scaled by an exact power of two, so that |b|^2 lies in [1, 8).
+__device__ __forceinline__ double2 cdiv1(double2 a, double2 b) {
+    const unsigned ex = unsigned(__double2hiint(b.x) >> 20) & 0x7FFu, ey = unsigned(__double2hiint(b.y) >> 20) & 0x7FFu;
+    const unsigned e = max(ex, ey);
+    if (e == 0u || e >= 0x7FEu) return cdiv(a, b);           // zero, subnormal, at the top of the range, not finite
+    const double s = __hiloint2double(int((0x7FEu - e) << 20), 0);         // 2^(1023 - e)
+    const double bx = b.x * s, by = b.y * s;
+    const double r = 1.0 / fma(bx, bx, by * by) * s;
+    return make_double2(fma(a.x, bx, a.y * by) * r, fma(a.y, bx, -a.x * by) * r);
+}
+
 // CUDA device sanity check used by every compute entry point.
 void require_device();
 msb_status guard(const char* fn, const std::function<void()>& body);

@@ -140,6 +140,8 @@ struct LzEpi {
     const double* qp;
     const double* bprev;
     double* part;
+    double* a_out;        // a_k, written by the last CTA
+    unsigned* cnt;
     double bp, dot;
     __device__ __forceinline__ bool stop() const { return false; }
     __device__ __forceinline__ void begin(int) { bp = bprev[0]; }
@@ -154,6 +156,9 @@ struct LzEpi {
         double acc[1] = {dot};
         block_sum_sm<1>(acc, sm);
         if (threadIdx.x == 0) part[blockIdx.x] = acc[0];
+        if (!last_cta(cnt, gridDim.x)) return;
+        sum_partials_cg<1>(part, gridDim.x, acc, sm);
+        if (threadIdx.x == 0) *a_out = acc[0];
     }
 };
 
@@ -166,51 +171,68 @@ __global__ void k_lz_sum(const double* part, int nblk, const int* cols, double* 
     if (threadIdx.x == 0) out[int64_t(k) * stride_k + c] = v[0];
 }
 
-// w -= a q; partial ||w||^2.
-template <typename V>
-__global__ void __launch_bounds__(256) k_lz_orth(const V* __restrict__ q, V* __restrict__ w, int64_t n,
-                                                 const int* __restrict__ cols, const double* __restrict__ a,
-                                                 double* part) {
-    __shared__ double sm[32];
-    const int c = cols[blockIdx.y];
-    const int64_t off = int64_t(c) * n;
-    const double ac = a[c];
-    double acc[1] = {0.0};
-    for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n;
-         s += int64_t(gridDim.x) * blockDim.x) {
-        const V x = vsub(w[off + s], cscale(ac, 0.0, q[off + s]));
-        w[off + s] = x;
-        acc[0] += norm2(x);
+// w -= a q; the last CTA: b = ||w||, stored for level k and as the current b.
+__global__ void __launch_bounds__(256) k_lz_orth(const double* __restrict__ q, double* __restrict__ w, int64_t n,
+                                                 const double* __restrict__ a, double* part, unsigned* cnt,
+                                                 double* b_out, double* bcur) {
+    __shared__ double sm[256];
+    const double ac = -a[0];
+    double acc[1] = {0.0}, acc2 = 0.0;
+    const int64_t h = n >> 1, nth = int64_t(gridDim.x) * blockDim.x;
+    const double2* __restrict__ q2 = reinterpret_cast<const double2*>(q);
+    double2* __restrict__ w2 = reinterpret_cast<double2*>(w);
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < h; i += nth) {
+        const double2 x = q2[i];
+        double2 y = w2[i];
+        y.x = fma(ac, x.x, y.x);
+        y.y = fma(ac, x.y, y.y);
+        w2[i] = y;
+        acc[0] = fma(y.x, y.x, acc[0]);
+        acc2 = fma(y.y, y.y, acc2);
     }
-    store_partials<1>(acc, sm, part);
-}
-
-// b_c = sqrt(sum); stores b[k][c] and the current b for the next step.
-__global__ void k_lz_norm(const double* part, int nblk, const int* cols, double* bstore, int64_t stride_k, int k,
-                          double* bcur) {
-    __shared__ double sm[32];
-    const int c = cols[blockIdx.x];
-    double v[1];
-    reduce_partials<1>(part + int64_t(blockIdx.x) * nblk, nblk, v, sm);
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+        const double y = fma(ac, q[n - 1], w[n - 1]);
+        w[n - 1] = y;
+        acc[0] = fma(y, y, acc[0]);
+    }
+    acc[0] += acc2;
+    block_sum_sm<1>(acc, sm);
+    if (threadIdx.x == 0) part[blockIdx.x] = acc[0];
+    if (!last_cta(cnt, gridDim.x)) return;
+    sum_partials_cg<1>(part, gridDim.x, acc, sm);
     if (threadIdx.x == 0) {
-        const double b = sqrt(v[0]);
-        bstore[int64_t(k) * stride_k + c] = b;
-        bcur[c] = b;
+        const double b = sqrt(acc[0]);
+        *b_out = b;
+        *bcur = b;
     }
 }
 
-// w *= 1/b (becomes q_{k+1}); a zero b leaves w (the column is finished).
-template <typename V>
-__global__ void __launch_bounds__(256) k_lz_scale(V* __restrict__ w, int64_t n, const int* __restrict__ cols,
-                                                  const double* __restrict__ bcur) {
-    const int c = cols[blockIdx.y];
-    const double b = bcur[c];
-    if (!(b > 0.0)) return;
-    const double inv = 1.0 / b;
-    const int64_t off = int64_t(c) * n;
-    for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n;
-         s += int64_t(gridDim.x) * blockDim.x)
-        w[off + s] = cscale(inv, 0.0, w[off + s]);
+// w *= 1/b (becomes q_{k+1}); a zero b leaves w (the Krylov space is exhausted).  g (or
+// null): also g += y q_{k+1}, the eigenvector's sum in the second pass.
+__global__ void __launch_bounds__(256) k_lz_scale(double* __restrict__ w, int64_t n, const double* __restrict__ bcur,
+                                                  double* __restrict__ g, double y) {
+    const double b = bcur[0];
+    const double inv = b > 0.0 ? 1.0 / b : 1.0;
+    const int64_t h = n >> 1, nth = int64_t(gridDim.x) * blockDim.x;
+    double2* __restrict__ w2 = reinterpret_cast<double2*>(w);
+    double2* __restrict__ g2 = reinterpret_cast<double2*>(g);
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < h; i += nth) {
+        double2 x = w2[i];
+        x.x *= inv;
+        x.y *= inv;
+        w2[i] = x;
+        if (g) {
+            double2 s = g2[i];
+            s.x = fma(y, x.x, s.x);
+            s.y = fma(y, x.y, s.y);
+            g2[i] = s;
+        }
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+        const double x = w[n - 1] * inv;
+        w[n - 1] = x;
+        if (g) g[n - 1] = fma(y, x, g[n - 1]);
+    }
 }
 
 // q_c = x_c / ||x_c|| (start vectors), norms n0[c] = <x_c|x_c>.
@@ -300,14 +322,15 @@ __global__ void k_scale_real(double* g, int64_t n, double f) {
 // sums per block.  Allocated by msb_ground_state, carved from a fixed array by
 // msb_ground_state_noalloc; the Lanczos run below is the same for both.
 struct GroundScratch {
-    double* Q;        // 3 n
+    double* Q;        // 3 ld
+    int64_t ld;       // vector stride: n rounded up to even (16-byte accesses)
     double* v0;       // n
     double* hbuf;     // n
     double* a;        // maxit + 1
     double* b;        // maxit + 1
     double* bcur;     // 1
     double* n0;       // 1
-    int* col0;        // 1
+    int* col0;        // 2: the column list (0), an arrival counter
     double* part;     // part_n partial sums: at least 3 per block, and one per CTA of the
     int part_n;       // row-tiled product
 };
@@ -320,7 +343,8 @@ static void lanczos_ground(const msb_op* op, const View& view, int64_t n, double
     RowPlan rows;
     if constexpr (std::is_same<View, HubView>::value) rows = row_plan<double>(op, 1);
     rows.ok = rows.ok && rows.grid <= S.part_n;
-    MSB_CUDA(cudaMemsetAsync(S.col0, 0, sizeof(int), st));
+    const int grid_o = std::min(grid, 4 * sm_count());
+    MSB_CUDA(cudaMemsetAsync(S.col0, 0, 2 * sizeof(int), st));
     if (start) MSB_CUDA(cudaMemcpyAsync(S.v0, start, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
     else { k_fill_start<<<grid, 256, 0, st>>>(S.v0, n, 0x5EEDull); ++out.launches; }
     std::vector<double> ha(maxit + 1), hb(maxit + 1), y;
@@ -328,39 +352,47 @@ static void lanczos_ground(const msb_op* op, const View& view, int64_t n, double
     // One Lanczos run from v0.  If `accumulate`, g = sum_i y[i] q_i.
     auto run = [&](int kmax, bool accumulate, int& k_done) {
         double* q = S.Q;
-        double* qp = S.Q + n;
-        double* w = S.Q + 2 * n;
+        double* qp = S.Q + S.ld;
+        double* w = S.Q + 2 * S.ld;
         k_lz_norm_partial<double><<<dim3(grid, 1), 256, 0, st>>>(S.v0, n, S.col0, S.part);
         k_lz_sum<<<1, 256, 0, st>>>(S.part, grid, S.col0, S.n0, 0, 0);
         k_lz_start<double><<<dim3(grid, 1), 256, 0, st>>>(S.v0, q, qp, n, S.col0, S.n0);
         MSB_CUDA(cudaMemsetAsync(S.bcur, 0, sizeof(double), st));
         out.launches += 3;
-        if (accumulate) MSB_CUDA(cudaMemsetAsync(g, 0, n * sizeof(double), st));
+        if (accumulate) {
+            MSB_CUDA(cudaMemsetAsync(g, 0, n * sizeof(double), st));
+            k_axpy_real<<<grid, 256, 0, st>>>(g, q, n, y[0]);
+            ++out.launches;
+        }
+        unsigned* cnt = reinterpret_cast<unsigned*>(S.col0 + 1);
+        const bool g16 = (reinterpret_cast<uintptr_t>(g) & 15u) == 0;     // the caller's vector
         int k = 0;
         for (; k < kmax; ++k) {
-            if (accumulate) { k_axpy_real<<<grid, 256, 0, st>>>(g, q, n, y[k]); ++out.launches; }
             if (accumulate && k == kmax - 1) break;
             {
                 ProfScope ps("ground_state", st, 3 * vb + op->matrix_bytes(8), hxf + 4.0 * n);
                 if (rows.ok)
-                    launch_hub_rows<double>(rows, nullptr, q, n, 1, 0.0, LzEpi{w, qp, S.bcur, S.part, 0.0, 0.0}, st);
+                    launch_hub_rows<double>(rows, nullptr, q, n, 1, 0.0,
+                                            LzEpi{w, qp, S.bcur, S.part, S.a + k, cnt, 0.0, 0.0}, st);
                 else
                     k_lz_apply<View, double><<<dim3(grid, 1), 256, 0, st>>>(view, q, qp, w, n, S.col0, S.bcur, S.part);
             }
-            {
+            if (!rows.ok) {
                 ProfScope ps("ground_state", st, 0, 0);
-                k_lz_sum<<<1, 256, 0, st>>>(S.part, rows.ok ? rows.grid : grid, S.col0, S.a, 1, k);
+                k_lz_sum<<<1, 256, 0, st>>>(S.part, grid, S.col0, S.a, 1, k);
+                ++out.launches;
             }
             {
                 ProfScope ps("ground_state", st, 3 * vb, 4.0 * n);
-                k_lz_orth<double><<<dim3(grid, 1), 256, 0, st>>>(q, w, n, S.col0, S.a + k, S.part);
+                k_lz_orth<<<grid_o, 256, 0, st>>>(q, w, n, S.a + k, S.part, cnt, S.b + k, S.bcur);
             }
-            { ProfScope ps("ground_state", st, 0, 0); k_lz_norm<<<1, 256, 0, st>>>(S.part, grid, S.col0, S.b, 1, k, S.bcur); }
             {
                 ProfScope ps("ground_state", st, 2 * vb, 1.0 * n);
-                k_lz_scale<double><<<dim3(grid, 1), 256, 0, st>>>(w, n, S.col0, S.bcur);
+                const bool acc = accumulate && g16;
+                k_lz_scale<<<grid_o, 256, 0, st>>>(w, n, S.bcur, acc ? g : nullptr, acc ? y[k + 1] : 0.0);
             }
-            out.launches += 5;
+            if (accumulate && !g16) { k_axpy_real<<<grid, 256, 0, st>>>(g, w, n, y[k + 1]); ++out.launches; }
+            out.launches += 3;
             ++out.matvecs;
             MSB_LAUNCH_CHECK();
             std::swap(qp, q);   // q_prev <- q
@@ -422,9 +454,10 @@ static void ground_state_impl(const msb_op* op, const View& view, int64_t n, dou
                               double* g, GroundResult& out, cudaStream_t st) {
     const int grid = grid_for(n, 256, 8);
     const int part_n = std::max(3 * grid, 4096);
-    DevBuf<double> Q(3 * size_t(n)), v0(n), hbuf(n), part(part_n), a_dev(maxit + 1), b_dev(maxit + 1), bcur(1), n0(1);
-    DevBuf<int> col0(1);
-    const GroundScratch S{Q.p, v0.p, hbuf.p, a_dev.p, b_dev.p, bcur.p, n0.p, col0.p, part.p, part_n};
+    const int64_t ld = (n + 1) / 2 * 2;
+    DevBuf<double> Q(3 * size_t(ld)), v0(n), hbuf(n), part(part_n), a_dev(maxit + 1), b_dev(maxit + 1), bcur(1), n0(1);
+    DevBuf<int> col0(2);
+    const GroundScratch S{Q.p, ld, v0.p, hbuf.p, a_dev.p, b_dev.p, bcur.p, n0.p, col0.p, part.p, part_n};
     lanczos_ground(op, view, n, tol, maxit, start, g, S, grid, out, st);
 }
 
@@ -447,19 +480,27 @@ void ground_state(msb_op* H, double tol, int maxit, const double* start, double*
 // convergent is carried forward: each call folds in levels [k_from, k_to) and
 // keeps the recurrence state per (column, w), so a run of K levels costs O(K)
 // per point instead of O(K^2 / check) for bottom-up re-evaluation at every check.
-// One CTA per active column; threads over w.  Also reports the column's
-// max |I_new - I_old| and max |I_new|.
+// One thread per (active column, w): blockIdx.x the column, blockIdx.y a block of w.  The
+// levels are a serial chain of two complex reciprocals, so the latency of a division
+// bounds it: one division per reciprocal (cdiv1), and no thread takes a second w.  The
+// column's max |I_new - I_old| and max |I_new| go to diff (zeroed by the caller) by an
+// integer maximum, which orders non-negative doubles.
+// Measured: 24 columns x 400 w, 60 levels 735 -> EVAL_NEW us.
 // ---------------------------------------------------------------------------
-__global__ void k_cf_eval(const double* __restrict__ a, const double* __restrict__ b, int64_t stride_k,
-                          const double* __restrict__ n0, const int* __restrict__ cols, int k_from, int k_to,
-                          const double* __restrict__ E0c, const double* __restrict__ w, int n_w, double eta,
-                          double2* __restrict__ gst, double2* __restrict__ Cst, double2* __restrict__ Dst,
-                          double* I, double* diff) {
-    __shared__ double sm[2 * 32];
+constexpr int kEvalThreads = 64;
+__global__ void __launch_bounds__(kEvalThreads) k_cf_eval(const double* __restrict__ a, const double* __restrict__ b,
+                                                          int64_t stride_k, const double* __restrict__ n0,
+                                                          const int* __restrict__ cols, int k_from, int k_to,
+                                                          const double* __restrict__ E0c, const double* __restrict__ w,
+                                                          int n_w, double eta, double2* __restrict__ gst,
+                                                          double2* __restrict__ Cst, double2* __restrict__ Dst, double* I,
+                                                          double* diff) {
     const int c = cols[blockIdx.x];
     const double E0 = E0c[c];
+    const int i = blockIdx.y * kEvalThreads + threadIdx.x;
     double dmax = 0.0, imax = 0.0;
-    for (int i = threadIdx.x; i < n_w; i += blockDim.x) {
+    if (i < n_w) {
+        const double2 one = make_double2(1.0, 0.0);
         const double2 z = make_double2(E0 + w[i], eta);
         const int64_t o = int64_t(c) * n_w + i;
         // g = d_0 + c_1 / (d_1 + c_2 / (d_2 + ...)), d_j = z - a_j, c_j = -b_j^2, by the
@@ -483,31 +524,25 @@ __global__ void k_cf_eval(const double* __restrict__ a, const double* __restrict
             const double bj = b[int64_t(j - 1) * stride_k + c];
             const double cj = -bj * bj;
             const double2 d = make_double2(z.x - aj, z.y);
-            D = cdiv(make_double2(1.0, 0.0), make_double2(fma(cj, D.x, d.x), fma(cj, D.y, d.y)));
-            const double2 ic = cdiv(make_double2(1.0, 0.0), C);
+            D = cdiv1(one, make_double2(fma(cj, D.x, d.x), fma(cj, D.y, d.y)));
+            const double2 ic = cdiv1(one, C);
             C = make_double2(fma(cj, ic.x, d.x), fma(cj, ic.y, d.y));
             g = cmul(g, cmul(C, D));
         }
         gst[o] = g;
         Cst[o] = C;
         Dst[o] = D;
-        const double2 G = cdiv(make_double2(1.0, 0.0), g);
+        const double2 G = cdiv1(one, g);
         const double val = k_to > 0 ? -(n0[c] * G.y) / M_PI : 0.0;
         dmax = fmax(dmax, fabs(val - I[o]));
         imax = fmax(imax, fabs(val));
         I[o] = val;
     }
-    // block max via sums of squares is not a max: do a shuffle max instead
     dmax = warp_max(dmax);
     imax = warp_max(imax);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if (lane == 0) { sm[wid] = dmax; sm[32 + wid] = imax; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double d = 0, m = 0;
-        for (int i = 0; i < nw; ++i) { d = fmax(d, sm[i]); m = fmax(m, sm[32 + i]); }
-        diff[2 * c] = d;
-        diff[2 * c + 1] = m;
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(reinterpret_cast<unsigned long long*>(diff + 2 * c), __double_as_longlong(dmax));
+        atomicMax(reinterpret_cast<unsigned long long*>(diff + 2 * c + 1), __double_as_longlong(imax));
     }
 }
 
@@ -530,6 +565,50 @@ struct CFCoef {
     float* cCf;
 };
 
+// End of pass A or B for columns of few CTAs: the column's last CTA adds its partial sums
+// and forms a_k (or b_{k+1}) itself, which saves a launch; cnt = null: the separate
+// kernels k_cf_reduce_a / _b (many CTAs per column, where the fence of every CTA costs
+// more than a launch).
+struct CFTail {
+    unsigned* cnt;        // arrival counter per column slot (blockIdx.y)
+    double* store;        // a or b, level-major
+    int64_t stride_k;
+    int k;
+};
+
+// a_k = sig_k * sum;  cC = a_k sig_k.
+__device__ __forceinline__ void cf_set_a(double sum, int c, double* store, int64_t stride_k, int k, const CFCoef& cf) {
+    const double a = cf.sig[c] * sum;
+    store[int64_t(k) * stride_k + c] = a;
+    cf.cC[c] = a * cf.sig[c];
+    cf.cCf[c] = float(cf.cC[c]);
+}
+
+// b_{k+1} = ||W||; next step: cB = b_{k+1} sig_k, sig = 1 / b_{k+1}.
+__device__ __forceinline__ void cf_set_b(double sum, int c, double* store, int64_t stride_k, int k, const CFCoef& cf) {
+    const double b = sqrt(sum);
+    store[int64_t(k) * stride_k + c] = b;
+    cf.cB[c] = b * cf.sig[c];
+    cf.sig[c] = b > 0.0 ? 1.0 / b : 0.0;
+    cf.cBf[c] = float(cf.cB[c]);
+    cf.sigf[c] = float(cf.sig[c]);
+}
+
+template <bool B>
+__device__ __forceinline__ void cf_tail(const CFTail& t, const double* part, int c, const CFCoef& cf) {
+    if (t.cnt == nullptr) return;
+    __shared__ double sm[32];
+    if (!last_cta(t.cnt + blockIdx.y, gridDim.x)) return;
+    double v[1] = {0.0};
+    const double* __restrict__ pc = part + int64_t(blockIdx.y) * gridDim.x;
+    for (int i = threadIdx.x; i < int(gridDim.x); i += blockDim.x) v[0] += __ldcg(pc + i);
+    block_sum<1>(v, sm);
+    if (threadIdx.x == 0) {
+        if (B) cf_set_b(v[0], c, t.store, t.stride_k, t.k, cf);
+        else cf_set_a(v[0], c, t.store, t.stride_k, t.k, cf);
+    }
+}
+
 constexpr int kMaxHops = 32;     // up-spin hops per row (a 2D 3 x 4 cluster has 24 bonds)
 
 // Pass A for the Hubbard operator, one CTA per (row u, active column): row u
@@ -547,7 +626,7 @@ template <typename C, bool Multi>
 __global__ void __launch_bounds__(256, 6) k_cf_apply_hub(HubView h0, const HubView* __restrict__ hv,
                                                          const int* __restrict__ colq, const C* __restrict__ Vk,
                                                          const C* __restrict__ Vkm1, C* __restrict__ W, int64_t ld,
-                                                         const int* __restrict__ cols, CFCoef cf, double* part) {
+                                                         const int* __restrict__ cols, CFCoef cf, double* part, CFTail tail) {
     using S = scalar_t<C>;
     const int c = cols[blockIdx.y];
     const int u = blockIdx.x;
@@ -555,6 +634,7 @@ __global__ void __launch_bounds__(256, 6) k_cf_apply_hub(HubView h0, const HubVi
     if constexpr (Multi) h = hv[colq[c]];
     if (Multi && u >= h.Dup) {            // row beyond this column's cluster
         if (threadIdx.x == 0) part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = 0.0;
+        cf_tail<false>(tail, part, c, cf);
         return;
     }
     const int L = h.L;
@@ -667,6 +747,7 @@ __global__ void __launch_bounds__(256, 6) k_cf_apply_hub(HubView h0, const HubVi
         block_sum<1>(acc, red);
         if (threadIdx.x == 0) part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = acc[0];
     }
+    cf_tail<false>(tail, part, c, cf);
 }
 
 // ---------------------------------------------------------------------------
@@ -708,13 +789,14 @@ __global__ void __launch_bounds__(256, 5) k_cf_apply_hub_fx(HubView h0, const Hu
                                                             const double2* __restrict__ Vk,
                                                             const double2* __restrict__ Vkm1,
                                                             double2* __restrict__ W, int64_t ld,
-                                                            const int* __restrict__ cols, CFCoef cf, double* part) {
+                                                            const int* __restrict__ cols, CFCoef cf, double* part, CFTail tail) {
     const int c = cols[blockIdx.y];
     const int u = blockIdx.x;
     HubView h = h0;
     if constexpr (Multi) h = hv[colq[c]];
     if (Multi && u >= h.Dup) {            // row beyond this column's cluster
         if (threadIdx.x == 0) part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = 0.0;
+        cf_tail<false>(tail, part, c, cf);
         return;
     }
     const int L = h.L;
@@ -830,6 +912,7 @@ __global__ void __launch_bounds__(256, 5) k_cf_apply_hub_fx(HubView h0, const Hu
     double acc[1] = {dot};
     block_sum<1>(acc, red);
     if (threadIdx.x == 0) part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = acc[0];
+    cf_tail<false>(tail, part, c, cf);
 }
 
 // FP32 pass A with two adjacent elements per thread (NT threads, MINB CTAs per SM:
@@ -849,13 +932,14 @@ __global__ void __launch_bounds__(NT, MINB) k_cf_apply_hub_f2x2(HubView h0, cons
                                                               const float2* __restrict__ Vk,
                                                               const float2* __restrict__ Vkm1, float2* __restrict__ W,
                                                               int64_t ld, const int* __restrict__ cols, CFCoef cf,
-                                                              double* part) {
+                                                              double* part, CFTail tail) {
     const int c = cols[blockIdx.y];
     const int u = blockIdx.x;
     HubView h = h0;
     if constexpr (Multi) h = hv[colq[c]];
     if (Multi && u >= h.Dup) {            // row beyond this column's cluster
         if (threadIdx.x == 0) part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = 0.0;
+        cf_tail<false>(tail, part, c, cf);
         return;
     }
     extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -999,6 +1083,7 @@ __global__ void __launch_bounds__(NT, MINB) k_cf_apply_hub_f2x2(HubView h0, cons
     }
     const double tot = block_sum_df(dhi, dlo, red);
     if (threadIdx.x == 0) part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = tot;
+    cf_tail<false>(tail, part, c, cf);
 }
 
 // The FP32 pass A for two columns per CTA (one operator for all columns): the two
@@ -1170,7 +1255,7 @@ __global__ void __launch_bounds__(256, 4) k_cf_apply_hub_f2x2c2(HubView h, const
 template <class View, typename C>
 __global__ void __launch_bounds__(256) k_cf_apply_gen(View op, const C* __restrict__ Vk, const C* __restrict__ Vkm1,
                                                       C* __restrict__ W, int64_t n, int64_t ld,
-                                                      const int* __restrict__ cols, CFCoef cf, double* part) {
+                                                      const int* __restrict__ cols, CFCoef cf, double* part, CFTail tail) {
     using S = scalar_t<C>;
     __shared__ double sm[32];
     const int c = cols[blockIdx.y];
@@ -1199,6 +1284,7 @@ __global__ void __launch_bounds__(256) k_cf_apply_gen(View op, const C* __restri
     if constexpr (std::is_same<S, float>::value) dot = df_value(dhi, dlo);
     double acc[1] = {dot};
     store_partials<1>(acc, sm, part);
+    cf_tail<false>(tail, part, c, cf);
 }
 
 // a_k = sig_k * sum;  cC = a_k sig_k.
@@ -1209,10 +1295,7 @@ __global__ void k_cf_reduce_a(const double* part, int nblk, const int* cols, dou
     double v[1];
     reduce_partials<1>(part + int64_t(blockIdx.x) * nblk, nblk, v, sm);
     if (threadIdx.x == 0) {
-        const double a = cf.sig[c] * v[0];
-        astore[int64_t(k) * stride_k + c] = a;
-        cf.cC[c] = a * cf.sig[c];
-        cf.cCf[c] = float(cf.cC[c]);
+        cf_set_a(v[0], c, astore, stride_k, k, cf);
     }
 }
 
@@ -1238,7 +1321,7 @@ __device__ __forceinline__ void orth_step(float4 v, float4& x, float m, double&,
 template <typename C>
 __global__ void __launch_bounds__(256) k_cf_orth(const C* __restrict__ Vk, C* __restrict__ W, int64_t ld,
                                                  const int* __restrict__ cols, const int64_t* __restrict__ clen,
-                                                 CFCoef cf, double* part) {
+                                                 CFCoef cf, double* part, CFTail tail) {
     using S = scalar_t<C>;
     using V16 = typename std::conditional<std::is_same<S, float>::value, float4, double2>::type;
     constexpr int per = sizeof(V16) / sizeof(C);     // complex elements per 16-byte load
@@ -1274,6 +1357,7 @@ __global__ void __launch_bounds__(256) k_cf_orth(const C* __restrict__ Vk, C* __
         double a1[1] = {acc};
         store_partials<1>(a1, sm, part);
     }
+    cf_tail<true>(tail, part, c, cf);
 }
 
 // b_{k+1} = ||W||; next step: cB = b_{k+1} sig_k, sig = 1 / b_{k+1}.
@@ -1284,12 +1368,7 @@ __global__ void k_cf_reduce_b(const double* part, int nblk, const int* cols, dou
     double v[1];
     reduce_partials<1>(part + int64_t(blockIdx.x) * nblk, nblk, v, sm);
     if (threadIdx.x == 0) {
-        const double b = sqrt(v[0]);
-        bstore[int64_t(k) * stride_k + c] = b;
-        cf.cB[c] = b * cf.sig[c];
-        cf.sig[c] = b > 0.0 ? 1.0 / b : 0.0;
-        cf.cBf[c] = float(cf.cB[c]);
-        cf.sigf[c] = float(cf.sig[c]);
+        cf_set_b(v[0], c, bstore, stride_k, k, cf);
     }
 }
 
@@ -1374,7 +1453,7 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
     int64_t hub_smem = 0;
     bool rows = false, pair = false, fx = false, sgn = false;
     int cpc = 1;                               // columns per CTA of the FP32 row-tiled apply
-    int fx_threads = 256;
+    int fx_threads = 256, f2_threads = kApplyThreads;
     int nblkA = grid;
     std::vector<HubView> hviews;
     if constexpr (hub) {
@@ -1408,6 +1487,12 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
             const int t = tuned_cf_threads(maxDdn, maxDup, MSB_FP64);
             if (t == 128 || t == 256) fx_threads = t;
         }
+        // Rows shorter than a CTA: no more threads than the row has elements (FP64) or pairs
+        // (FP32), in whole warps.  Half of a 256-thread CTA idles on the L = 10 ring's rows of
+        // 126 pairs (160 columns, per level 143 -> F2_NOTE us).  The warps keep their positions,
+        // so the placement and the hop schedule hold.
+        if (maxDdn < 128) fx_threads = int((maxDdn + 31) / 32 * 32);
+        if (maxDdn / 2 < kApplyThreads) f2_threads = int(std::max<int64_t>(1, (maxDdn / 2 + 31) / 32) * 32);
         // FP32 shape: 1 = one column per CTA at 6 CTAs per SM; 2 = two columns per CTA
         // (half the index work, 4 CTAs per SM); 3 = one column at 8 CTAs per SM (32
         // registers); 4 = one column per 512-thread CTA, 4 per SM (32 registers).
@@ -1492,7 +1577,12 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
     // L1/shared pipe) overlaps the orth pass of the other (bound by DRAM).  Each group's
     // levels are ordered on its own stream; the groups meet at every convergence check.
     // With the profiler on, one group, so that every launch is timed alone.
-    const int ngrp = prof_on() ? 1 : 2;
+    // Small batches take one group: a level is then two launches long, not bound by the
+    // pipes, and a second stream only doubles the launches (map of the L = 8 ring, 41
+    // columns of 4,900: MAPL8_NOTE).
+    const int ngrp = prof_on() || all_elems < 4e6 ? 1 : 2;
+    // a column's sums close in its own last CTA where the CTAs per column are few
+    const bool tails = cpc != 2 && nblkA <= 512;
     cudaStream_t gs[2] = {st, nullptr};
     cudaEvent_t gev = nullptr;
     if (ngrp == 2) {
@@ -1505,6 +1595,8 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
     } sguard{gs[1], gev};
     DevBuf<int> gcols_d[2];
     DevBuf<double> gpart[2];
+    DevBuf<unsigned> gcnt(2 * size_t(nv));
+    gcnt.zero(st);
     std::vector<int> gcols[2];
     for (int g = 0; g < ngrp; ++g) {
         gcols_d[g].alloc(std::max(nv, 1));
@@ -1541,6 +1633,12 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
         cudaStream_t s = gs[g];
         const int* cl = gcols_d[g].p;
         double* pt = gpart[g].p;
+        unsigned* cnt = tails ? gcnt.p + size_t(g) * nv : nullptr;
+        const CFTail ta{cnt, a.p, nv, kk}, tb{cnt, b.p, nv, kk};
+        // CTAs per column of the orth pass: about 16 per SM over all columns, with at least
+        // four 16-byte accesses per thread (thinner CTAs pay their block sum too often)
+        const int go = int(std::max<int64_t>(
+            1, std::min<int64_t>({int64_t(grid), (int64_t(sm_count()) * 16 + na - 1) / na, (ld / per + 1023) / 1024})));
         {
             ProfScope ps("cf_apply", s, grp_bytes[g], grp_flops[g]);
             bool done_hub = false;
@@ -1552,7 +1650,7 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
                     auto y = reinterpret_cast<double2*>(wv);
                     auto kern = multi ? (sgn ? k_cf_apply_hub_fx<true, true> : k_cf_apply_hub_fx<true, false>)
                                       : (sgn ? k_cf_apply_hub_fx<false, true> : k_cf_apply_hub_fx<false, false>);
-                    kern<<<gg, fx_threads, hub_smem, s>>>(view, hv.p, colq.p, x, xm, y, ld, cl, cf, pt);
+                    kern<<<gg, fx_threads, hub_smem, s>>>(view, hv.p, colq.p, x, xm, y, ld, cl, cf, pt, ta);
                     done_hub = true;
                 } else if (rows && pair && cpc == 2) {
                     auto x = reinterpret_cast<const float2*>(vk);
@@ -1571,38 +1669,37 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
                                 : cpc == 3 ? (sgn ? k_cf_apply_hub_f2x2<false, true, 8> : k_cf_apply_hub_f2x2<false, false, 8>)
                                 : multi    ? (sgn ? k_cf_apply_hub_f2x2<true, true, 6> : k_cf_apply_hub_f2x2<true, false, 6>)
                                            : (sgn ? k_cf_apply_hub_f2x2<false, true, 6> : k_cf_apply_hub_f2x2<false, false, 6>);
-                    kern<<<gg, cpc == 4 ? 512 : kApplyThreads, hub_smem, s>>>(view, hv.p, colq.p, x, xm, y, ld, cl, cf,
-                                                                            pt);
+                    kern<<<gg, cpc == 4 ? 512 : f2_threads, hub_smem, s>>>(view, hv.p, colq.p, x, xm, y, ld, cl, cf, pt, ta);
                     done_hub = true;
                 } else if (rows) {
                     // FP32 with an odd D_dn (FP64 always takes the fixed-point kernel)
                     if constexpr (std::is_same<C, float2>::value) {
                         if (multi)
                             k_cf_apply_hub<C, true><<<gg, kApplyThreads, hub_smem, s>>>(view, hv.p, colq.p, vk, vkm1,
-                                                                                         wv, ld, cl, cf, pt);
+                                                                                         wv, ld, cl, cf, pt, ta);
                         else
                             k_cf_apply_hub<C, false><<<gg, kApplyThreads, hub_smem, s>>>(view, hv.p, colq.p, vk, vkm1,
-                                                                                          wv, ld, cl, cf, pt);
+                                                                                          wv, ld, cl, cf, pt, ta);
                         done_hub = true;
                     }
                 }
             }
             if (!done_hub)
-                k_cf_apply_gen<View, C><<<dim3(grid, na), 256, 0, s>>>(view, vk, vkm1, wv, nlen[0], ld, cl, cf, pt);
+                k_cf_apply_gen<View, C><<<dim3(grid, na), 256, 0, s>>>(view, vk, vkm1, wv, nlen[0], ld, cl, cf, pt, ta);
         }
-        {
+        if (!tails) {
             ProfScope ps("cf_reduce", s, 0, 0);
             k_cf_reduce_a<<<na, 256, 0, s>>>(pt, rows ? nblkA : grid, cl, a.p, nv, kk, cf);
         }
         {
             ProfScope ps("cf_orth", s, 3.0 * grp_elems[g] * sizeof(C), 8.0 * grp_elems[g]);
-            k_cf_orth<C><<<dim3(grid, na), 256, 0, s>>>(vk, wv, ld, cl, clen_d.p, cf, pt);
+            k_cf_orth<C><<<dim3(go, na), 256, 0, s>>>(vk, wv, ld, cl, clen_d.p, cf, pt, tb);
         }
-        {
+        if (!tails) {
             ProfScope ps("cf_reduce", s, 0, 0);
-            k_cf_reduce_b<<<na, 256, 0, s>>>(pt, grid, cl, b.p, nv, kk, cf);
+            k_cf_reduce_b<<<na, 256, 0, s>>>(pt, go, cl, b.p, nv, kk, cf);
         }
-        out.launches += 4;
+        out.launches += tails ? 2 : 4;
         out.matvecs += na;
     };
     int k = 0;
@@ -1624,7 +1721,8 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
             cols.upload(hcols.data(), std::max(nact, 1), st);
             {
                 ProfScope ps("cf_eval", st, 0, 40.0 * nact * n_w * double(k - k_eval));
-                k_cf_eval<<<nact, 128, 0, st>>>(a.p, b.p, nv, n0.p, cols.p, k_eval, k, E0d.p, wdev.p, n_w, eta,
+                MSB_CUDA(cudaMemsetAsync(diff.p, 0, diff.bytes(), st));
+                k_cf_eval<<<dim3(nact, (n_w + kEvalThreads - 1) / kEvalThreads), kEvalThreads, 0, st>>>(a.p, b.p, nv, n0.p, cols.p, k_eval, k, E0d.p, wdev.p, n_w, eta,
                                                 gst.p, Cst.p, Dst.p, I.p, diff.p);
                 k_eval = k;
             }
@@ -1774,10 +1872,11 @@ static void ground_state_noalloc_impl(const msb_op* op, const View& view, int64_
     MSB_REQUIRE(grid <= kNoAllocMaxGrid, "grid exceeds the no-alloc scratch layout");
     double* base = noalloc_scratch_address();
     GroundScratch S;
-    S.Q = base;                               // 3 Lanczos vectors
-    S.v0 = base + 3 * n;                      // start vector of the current restart
-    S.hbuf = base + 4 * n;                    // H g for the residual check
-    S.a = base + 5 * n;                       // a_k
+    S.Q = base;                               // 3 Lanczos vectors, each of even length
+    S.ld = (n + 1) / 2 * 2;
+    S.v0 = base + 3 * S.ld;                   // start vector of the current restart
+    S.hbuf = S.v0 + S.ld;                     // H g for the residual check
+    S.a = S.hbuf + S.ld;                      // a_k
     S.b = S.a + (maxit + 1);                  // b_{k+1}
     S.bcur = S.b + (maxit + 1);
     S.n0 = S.bcur + 1;

@@ -50,7 +50,7 @@
 namespace msb {
 
 constexpr int kScalarThreads = 256;
-constexpr int kVecThreads = 512;      // vector kernels of the iteration, two CTAs per SM
+constexpr int kVecThreads = 256;      // vector kernels of the iteration, three CTAs per SM
 
 // ---------------------------------------------------------------------------
 // Device state
@@ -58,10 +58,11 @@ constexpr int kVecThreads = 512;      // vector kernels of the iteration, two CT
 struct SeedState {
     double2 rho;          // rho_m = (r_m, r_m)
     double2 alpha;        // alpha_m of the current iteration
-    double2 alpha_prev;   // alpha_{m-1} (1 before the first iteration)
     double2 beta;         // beta_m: built p_m (0 at m = 0)
     double2 beta_n, rho_n;   // beta_{m+1}, (r~_{m+1}, r~_{m+1}) before the rescale
-    double rn_n;          // ||r~_{m+1}||
+    double rn2_n;         // ||r~_{m+1}||^2
+    double2 irho;         // 1 / rho_m
+    double2 boa;          // beta_m / alpha_{m-1}
     int f_n, bad_n;       // its rescale exponent; why beta could not be formed
     unsigned cnt_a, cnt_b;   // arrival counters of the two reductions
     double rnorm;         // ||r_m||
@@ -100,16 +101,6 @@ struct SeedState {
 // 85 us for the two vector kernels at L = 12, as much as with separate scalar kernels).
 // ---------------------------------------------------------------------------
 
-// a / b with one division: b scaled by an exact power of two, so that |b|^2 lies in [1, 8).
-__device__ __forceinline__ double2 cdiv1(double2 a, double2 b) {
-    const unsigned ex = unsigned(__double2hiint(b.x) >> 20) & 0x7FFu, ey = unsigned(__double2hiint(b.y) >> 20) & 0x7FFu;
-    const unsigned e = max(ex, ey);
-    if (e == 0u || e >= 0x7FEu) return cdiv(a, b);           // zero, subnormal, at the top of the range, not finite
-    const double s = __hiloint2double(int((0x7FEu - e) << 20), 0);         // 2^(1023 - e)
-    const double bx = b.x * s, by = b.y * s;
-    const double r = 1.0 / fma(bx, bx, by * by) * s;
-    return make_double2(fma(a.x, bx, a.y * by) * r, fma(a.y, bx, -a.x * by) * r);
-}
 // x 2^n, exact while the result is a normal number.
 __device__ __forceinline__ double scale2(double x, int n) {
     return n > -1022 && n < 1023 ? x * __hiloint2double((1023 + n) << 20, 0) : ldexp(x, n);
@@ -190,7 +181,7 @@ struct MvmEpi {
     SeedState* st;
     double* part;
     const V* pt;
-    double c0r, c0i;
+    scalar_t<V> c0r, c0i;
     double acc[2];
     DF4 df;
     __device__ __forceinline__ bool stop() const { return mvm_halted(st); }
@@ -242,7 +233,7 @@ template <typename C>
 __device__ __forceinline__ void shift_scalars_a(SeedState* st, double2 alpha, const ShiftArrays& sh, int ns, int B) {
     if (threadIdx.x >= ns) return;
     const double2 beta = st->beta;
-    const double2 ab_over = cdiv1(cmul(alpha, beta), st->alpha_prev);   // alpha_m beta_m / alpha_{m-1}
+    const double2 ab_over = cmul(alpha, st->boa);                       // alpha_m beta_m / alpha_{m-1}
     const int j = st->j;
     const int fexp = st->fexp;
     for (int k = threadIdx.x; k < ns; k += blockDim.x) {
@@ -318,7 +309,7 @@ __device__ __forceinline__ float2 axpy_rn(float2 r, float2 c, float2 v, float sg
 // Bound by memory (three vectors; L2 while they fit); 16-byte accesses, two elements
 // per access in FP32, two accesses in flight per vector.
 template <typename V>
-__global__ void __launch_bounds__(kVecThreads) k_seed_update(V* ring, int64_t ld, const V* __restrict__ v, int64_t n,
+__global__ void __launch_bounds__(kVecThreads, 3) k_seed_update(V* ring, int64_t ld, const V* __restrict__ v, int64_t n,
                                                              int nslot, SeedState* __restrict__ st, double* part,
                                                              V* __restrict__ rt, const V* __restrict__ vt,
                                                              ShiftArrays sh, int ns, int B) {
@@ -409,24 +400,23 @@ __global__ void __launch_bounds__(kVecThreads) k_seed_update(V* ring, int64_t ld
     sum_partials_cg<3>(part, gridDim.x - 1, acc, sm);
     if (threadIdx.x == 0) {
         const double2 rho_new = make_double2(acc[0], acc[1]);
-        const double rnew = sqrt(acc[2]);
         double2 b = make_double2(0.0, 0.0);
         int bad = MSB_OK, f = 0;
-        if (!cfinite(rho_new) || !isfinite(rnew)) {
+        if (!cfinite(rho_new) || !isfinite(acc[2])) {
             bad = MSB_ENONFINITE;
-        } else if (rnew == 0.0) {
+        } else if (acc[2] == 0.0) {
             // exact solution: every shift converged
         } else if (rho_new.x == 0.0 && rho_new.y == 0.0) {
             bad = MSB_EBREAKDOWN;                           // (r, r) = 0 with r != 0
         } else {
-            b = cdiv1(rho_new, st->rho);
+            b = cmul(rho_new, st->irho);
             // bring ||r~|| back near ||b|| once it drifts by more than 2^20
-            const double ratio = rnew / st->bnorm;
-            if (ratio < 0x1p-20 || ratio > 0x1p20) f = -ilogb(ratio);
+            const double ratio2 = acc[2] * st->ibnorm * st->ibnorm;
+            if (ratio2 < 0x1p-40 || ratio2 > 0x1p40) f = -(ilogb(ratio2) >> 1);
         }
         st->beta_n = b;
         st->rho_n = rho_new;
-        st->rn_n = rnew;
+        st->rn2_n = acc[2];
         st->f_n = f;
         st->bad_n = bad;
     }
@@ -437,7 +427,7 @@ __global__ void __launch_bounds__(kVecThreads) k_seed_update(V* ring, int64_t ld
 // shift's recursive residual.
 __device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays& sh, int ns, int nslot, int* s_still) {
     const int m = st->m + 1, f = st->f_n, bad = st->bad_n;
-    const double rn = st->rn_n;
+    const double rn = sqrt(st->rn2_n);
     if (threadIdx.x == 0) *s_still = 0;
     __syncthreads();
     if (threadIdx.x < ns) {
@@ -464,9 +454,12 @@ __device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays
         st->m = m;
         st->j = st->jcur + 1;
         st->rexp[(st->slot0 + st->jcur + 1) % nslot] = rn > 0.0 && isfinite(rn) ? ilogb(rn) + f : 0;
-        st->alpha_prev = st->alpha;
+        // the divisions of the next iteration's scalars, off its critical path
+        const double2 rho = scale2(st->rho_n, 2 * f);
+        st->boa = cdiv1(st->beta_n, st->alpha);
+        st->irho = cdiv1(make_double2(1.0, 0.0), rho);
         st->beta = st->beta_n;
-        st->rho = scale2(st->rho_n, 2 * f);
+        st->rho = rho;
         st->rnorm = scale2(rn, -st->sexp);
         st->fexp = f;
         st->sexp += f;
@@ -480,7 +473,7 @@ __device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays
 // CTA 0: the per-shift convergence tests.
 // Dual form (rt != null): also p~ = 2^f (r~ + conj(beta) p~), r~ <- 2^f r~.
 template <typename V>
-__global__ void __launch_bounds__(kVecThreads) k_update_p(V* ring, int64_t ld, V* __restrict__ p, int64_t n, int nslot,
+__global__ void __launch_bounds__(kVecThreads, 3) k_update_p(V* ring, int64_t ld, V* __restrict__ p, int64_t n, int nslot,
                                                           SeedState* __restrict__ st, V* __restrict__ rt,
                                                           V* __restrict__ pt, ShiftArrays sh, int ns) {
     if (st->halted) return;
@@ -557,19 +550,28 @@ __global__ void k_block_begin(SeedState* st, ShiftArrays sh, int ns, int nslot) 
 // registers.  The order of the operations does not depend on the window.
 // Optional row map: element e of the per-shift vectors is seed element
 // rows[e / rowlen] * rowlen + e % rowlen (only the rows the caller needs).
-// FP32 (BMAX = 32, the whole window in one pass): with 16 FMAs per 8 bytes of r and 256
-// per 32 bytes of P and x, the FP32 pipe and DRAM are about balanced; the next shift's P
-// and x are loaded before the current one's arithmetic.  Measured (48 shifts, n = 2.9 M,
-// against a window of 8): see the FP32 solve in the commit that brought it.
-// FP64: bound by the FP64 pipe (8 FMAs per shift, element and iteration); windows with many
-// shifts go to the tensor cores (flush_tc.cuh), and this kernel returns at once.
-template <typename V, int BMAX>
-__global__ void __launch_bounds__(256, 2) k_flush(const V* __restrict__ ring, int nslot, int64_t ld,
-                                                  V* __restrict__ P, V* __restrict__ X, int64_t n_out,
-                                                  const int32_t* __restrict__ rows, int64_t rowlen,
-                                                  ShiftArrays sh, int ns, SeedState* __restrict__ st, int W,
-                                                  const int* __restrict__ tc_cnt) {
+// A thread carries NE elements: 2 NE FMAs per component pair share one coefficient load,
+// and the NE chains cover each other's latency.  The next shift's P and x are loaded before
+// the current one's arithmetic.
+// FP32 (BMAX = 32: the whole window in one pass; NE = 2, the 64 residuals in registers at
+// one CTA per SM): the FP32 pipe and DRAM are about balanced at 256 FMAs per 32 bytes of P
+// and x.  48 shifts, n = 2.9 M, per 32 iterations: 3.4 ms as four windows of 8, 2.5 ms with
+// NE = 1 (bound by the coefficient loads), MEASURED_NE2 with NE = 2.
+// FP64 (BMAX = 8, NE = 1): bound by the FP64 pipe (8 FMAs per shift, element and
+// iteration); windows with many shifts go to the tensor cores (flush_tc.cuh), and this
+// kernel returns at once.
+// (gamma, c) of one iteration, read in one access.
+template <typename V>
+struct __align__(16) CoefPair { V g, c; };
+
+template <typename V, int BMAX, int NE>
+__global__ void __launch_bounds__(256, NE == 1 ? 2 : 1) k_flush(const V* __restrict__ ring, int nslot, int64_t ld,
+                                                                V* __restrict__ P, V* __restrict__ X, int64_t n_out,
+                                                                const int32_t* __restrict__ rows, int64_t rowlen,
+                                                                ShiftArrays sh, int ns, SeedState* __restrict__ st,
+                                                                int W, const int* __restrict__ tc_cnt) {
     __shared__ int s_list[kMaxShifts];
+    __shared__ unsigned char s_J[kMaxShifts];
     __shared__ int s_cnt;
     const bool tc = tc_cnt != nullptr && tc_use(*tc_cnt, st->bnorm);
     if (tc && blockIdx.x != 0) return;
@@ -582,54 +584,84 @@ __global__ void __launch_bounds__(256, 2) k_flush(const V* __restrict__ ring, in
         st->flush_first = first;
     }
     if (tc || cnt == 0) return;
-    const V* __restrict__ coef = reinterpret_cast<const V*>(sh.coefv);
-    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < n_out;
-         e += int64_t(gridDim.x) * blockDim.x) {
-        int64_t src = e;
-        if (rows) {
-            const int64_t row = e / rowlen;
-            src = int64_t(__ldg(rows + row)) * rowlen + (e - row * rowlen);
+    for (int q = threadIdx.x; q < cnt; q += blockDim.x) s_J[q] = static_cast<unsigned char>(sh.nblk[s_list[q]]);
+    __syncthreads();
+    const CoefPair<V>* __restrict__ coef = reinterpret_cast<const CoefPair<V>*>(sh.coefv);
+    // element u of a thread: e + u * blockDim.x (whole lines for any n_out)
+    for (int64_t e = int64_t(blockIdx.x) * blockDim.x * NE + threadIdx.x; e < n_out;
+         e += int64_t(gridDim.x) * blockDim.x * NE) {
+        int64_t src[NE];
+        bool on[NE];
+#pragma unroll
+        for (int u = 0; u < NE; ++u) {
+            const int64_t eu = e + u * int64_t(blockDim.x);
+            on[u] = eu < n_out;
+            src[u] = on[u] ? eu : e;
+            if (rows) {
+                const int64_t row = src[u] / rowlen;
+                src[u] = int64_t(__ldg(rows + row)) * rowlen + (src[u] - row * rowlen);
+            }
         }
         for (int i0 = 0; i0 < JW; i0 += BMAX) {
             const bool fresh = first && i0 == 0;
-            V r[BMAX];
+            V r[NE][BMAX];
 #pragma unroll
             for (int i = 0; i < BMAX; ++i) {
                 const int sl = (slot0 + i0 + i) % nslot;
-                r[i] = (i0 + i < JW) ? ring[int64_t(sl) * ld + src] : vzero(V{});
+#pragma unroll
+                for (int u = 0; u < NE; ++u) r[u][i] = (i0 + i < JW) ? ring[int64_t(sl) * ld + src[u]] : vzero(V{});
             }
+            V np[NE], nx[NE];
+            auto fetch = [&](int k) {
+#pragma unroll
+                for (int u = 0; u < NE; ++u) {
+                    const int64_t o = int64_t(k) * n_out + e + u * int64_t(blockDim.x);
+                    np[u] = !fresh && on[u] ? P[o] : vzero(V{});
+                    nx[u] = !fresh && on[u] ? X[o] : vzero(V{});
+                }
+            };
             int k = s_list[0];
-            V np = fresh ? vzero(V{}) : P[int64_t(k) * n_out + e];
-            V nx = fresh ? vzero(V{}) : X[int64_t(k) * n_out + e];
+            fetch(k);
             for (int q = 0; q < cnt; ++q) {
                 const int kc = k;
-                V pk = np, xk = nx;
+                V pk[NE], xk[NE];
+#pragma unroll
+                for (int u = 0; u < NE; ++u) {
+                    pk[u] = np[u];
+                    xk[u] = nx[u];
+                }
                 if (q + 1 < cnt) {
                     k = s_list[q + 1];
-                    if (!fresh) {
-                        np = P[int64_t(k) * n_out + e];
-                        nx = X[int64_t(k) * n_out + e];
-                    }
+                    fetch(k);
                 }
-                const int J = sh.nblk[kc] - i0;
+                const int J = s_J[q] - i0;
                 if (J <= 0) continue;
-                const V* __restrict__ ck = coef + (int64_t(kc) * W + i0) * 2;
+                const CoefPair<V>* __restrict__ ck = coef + int64_t(kc) * W + i0;
+                auto step = [&](int i) {
+                    const CoefPair<V> gc = ck[i];
+#pragma unroll
+                    for (int u = 0; u < NE; ++u) {
+                        pk[u] = cfma(gc.g, pk[u], r[u][i]);        // P = r_i + gamma_i P
+                        xk[u] = cfma(gc.c, pk[u], xk[u]);          // x = x + c_i P
+                    }
+                };
                 if (J >= BMAX) {
 #pragma unroll
-                    for (int i = 0; i < BMAX; ++i) {
-                        pk = cfma(ck[2 * i], pk, r[i]);        // P = r_i + gamma_i P
-                        xk = cfma(ck[2 * i + 1], pk, xk);      // x = x + c_i P
-                    }
+                    for (int i = 0; i < BMAX; ++i) step(i);
                 } else {
 #pragma unroll
                     for (int i = 0; i < BMAX; ++i) {
                         if (i >= J) break;
-                        pk = cfma(ck[2 * i], pk, r[i]);
-                        xk = cfma(ck[2 * i + 1], pk, xk);
+                        step(i);
                     }
                 }
-                P[int64_t(kc) * n_out + e] = pk;
-                X[int64_t(kc) * n_out + e] = xk;
+#pragma unroll
+                for (int u = 0; u < NE; ++u) {
+                    if (!on[u]) continue;
+                    const int64_t o = int64_t(kc) * n_out + e + u * int64_t(blockDim.x);
+                    P[o] = pk[u];
+                    X[o] = xk[u];
+                }
             }
         }
     }
@@ -713,7 +745,8 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         const double bn = sqrt(v[2]);
         st->rho = make_double2(v[0], v[1]);
         st->alpha = make_double2(1.0, 0.0);
-        st->alpha_prev = make_double2(1.0, 0.0);
+        st->boa = make_double2(0.0, 0.0);
+        st->irho = cdiv1(make_double2(1.0, 0.0), st->rho);
         st->beta = make_double2(0.0, 0.0);
         st->rnorm = bn;
         st->bnorm = bn;
@@ -807,7 +840,8 @@ struct SolverImpl {
             ProfScope ps("seed_mvm", st, 2 * nb + op->matrix_bytes(csz), op->hx_flops() + 16.0 * n);
             if (rows.ok)
                 launch_hub_rows<V>(rows, rparts, p.p, n, 1, pr.c0.x,
-                                   MvmEpi<V>{v.p, state.p, part.p, pt.p, pr.c0.x, pr.c0.y, {0.0, 0.0}, {}}, st);
+                                   MvmEpi<V>{v.p, state.p, part.p, pt.p, scalar_t<V>(pr.c0.x), scalar_t<V>(pr.c0.y),
+                                             {0.0, 0.0}, {}}, st);
             else
                 k_mvm_dot<View, V><<<grid_vec, 256, 0, st>>>(view, p.p, v.p, n, pr.c0.x, pr.c0.y, state.p, part.p, pt.p);
         }
@@ -836,8 +870,8 @@ struct SolverImpl {
                 k_tc_coef<<<(pr.ns + 3) / 4, 128, 0, st>>>(nblk.p, coef64.p, pr.ns, W, nslot, &state.p->slot0,
                                                           &state.p->bnorm, tcc);
             }
-            constexpr int BMAX = std::is_same<V, float2>::value ? 32 : 8;
-            k_flush<V, BMAX><<<grid_flush, 256, 0, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, pr.rows, pr.rowlen,
+            constexpr int BMAX = std::is_same<V, float2>::value ? 32 : 8, NE = std::is_same<V, float2>::value ? 2 : 1;
+            k_flush<V, BMAX, NE><<<grid_flush, 256, 0, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, pr.rows, pr.rowlen,
                                                          sh, pr.ns, state.p, W, cnt);
             if constexpr (std::is_same<V, double2>::value) {
                 if (tc)
@@ -865,13 +899,13 @@ struct SolverImpl {
         B = pr.block;
         W = std::is_same<V, float2>::value ? 32 : kTcWindow;
         grid_vec = grid_for(n, 256, 8);
-        grid_flush = grid_for(pr.n_out, 256, 8);
+        grid_flush = std::is_same<V, float2>::value ? grid_for((pr.n_out + 1) / 2, 256, 4) : grid_for(pr.n_out, 256, 8);
         constexpr bool f32 = std::is_same<V, float2>::value;
         rows = op->kind == 2 ? (f32 ? op->plan32 : op->plan64) : row_plan<V>(op, 1);
         if (op->kind == 2) rparts = f32 ? op->parts32.p : op->parts64.p;
         grid_mvm = rows.ok ? rows.grid : grid_vec;
         ld = (n + 1) / 2 * 2;
-        grid_upd = grid_for((n * int64_t(sizeof(V)) + 15) / 16, kVecThreads, 2);
+        grid_upd = std::min(grid_for((n * int64_t(sizeof(V)) + 15) / 16, kVecThreads, 3), 3 * sm_count() - 1);
         if (size_t(W + 1) * ld * sizeof(V) > (size_t(16) << 30)) W = B;
         try {
             ring.alloc(size_t(W + 1) * ld);

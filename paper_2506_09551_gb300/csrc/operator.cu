@@ -224,7 +224,7 @@ template <typename V>
 struct ApplyEpi {
     V* y;
     int64_t n;
-    double c0r, c0i;
+    scalar_t<V> c0r, c0i;       // in the vector's precision: no FP64 conversion per element
     __device__ __forceinline__ bool stop() const { return false; }
     __device__ __forceinline__ void begin(int col) { y += int64_t(col) * n; }
     template <typename S>
@@ -249,7 +249,7 @@ static bool launch_apply_rows(const msb_op* op, double2 c0, const void* x, void*
     const int64_t n = op->dim;
     ProfScope ps("h_apply", st, nvec * 2.0 * n * sizeof(V), nvec * (op->hx_flops() + 8.0 * n));
     launch_hub_rows<V>(p, op->kind == 2 ? (f32 ? op->parts32.p : op->parts64.p) : nullptr, (const V*)x, n, nvec, c0.x,
-                       ApplyEpi<V>{(V*)y, n, c0.x, c0.y}, st);
+                       ApplyEpi<V>{(V*)y, n, scalar_t<V>(c0.x), scalar_t<V>(c0.y)}, st);
     MSB_LAUNCH_CHECK();
     count_launch();
     return true;
