@@ -118,15 +118,13 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
         }
         for (int i = threadIdx.x; i < 3 * (L + 1); i += nt) {
             const int nb = i / (L + 1), pc = i - nb * (L + 1);
-            // FP64: c0's real part and the block's shift are folded into the diagonal, which saves
-            // two FP64 operations per element at the same rounding error.  FP32: they stay
-            // apart, since the sum rounded to 32 bits would perturb the operator.
-            if constexpr (sizeof(S) == 8) lut[i] = h.U * double(pc) - h.Uc * double(nb) + P.shift + c0r;
+            if constexpr (sizeof(S) == 8) lut[i] = h.U * double(pc) - h.Uc * double(nb);
             else lut[i] = h.Uf * float(pc) - h.Ucf * float(nb);
         }
         __syncthreads();
         const int core = h.core;
-        const S mt = S(-h.t), shift = S(P.shift);
+        // FP64: the block's shift and the real part of c0 as one constant (c0 alone without a sum)
+        const S mt = S(-h.t), shift = sizeof(S) == 8 ? S(P.shift + c0r) : S(P.shift);
         const S s1 = S(one);                                       // 1, opaque to the compiler: an FMA, not an add
         const uint16_t* __restrict__ t16 = h.hdnr16;
         constexpr int PE = PAIR ? 2 : 1;
@@ -238,10 +236,13 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
     epi.finish(red);
 }
 
-// H x + c0 x from the hop sum and the diagonal.  FP64: the real part of c0 and the shift
-// are in dg.  FP32: added here, in the order of the element-wise kernels.
-__device__ __forceinline__ double2 hub_value(double2 acc, double dg, double mt, double, double, double c0i, double2 x) {
-    return make_double2(fma(mt, acc.x, fma(dg, x.x, -c0i * x.y)), fma(mt, acc.y, fma(dg, x.y, c0i * x.x)));
+// H x + c0 x from the hop sum and the diagonal.  FP64: `shift` holds the real part of c0 too;
+// it is not folded into the diagonal, whose sum with it would be rounded at the diagonal's
+// size (eight vectors at L = 12: distance from the 64-bit reference 4.3e-17 with the
+// element-wise kernel, 9.6e-17 folded).  FP32: in the order of the element-wise kernels.
+__device__ __forceinline__ double2 hub_value(double2 acc, double dg, double mt, double shift, double, double c0i, double2 x) {
+    return make_double2(fma(mt, acc.x, fma(dg, x.x, fma(shift, x.x, -c0i * x.y))),
+                        fma(mt, acc.y, fma(dg, x.y, fma(shift, x.y, c0i * x.x))));
 }
 __device__ __forceinline__ float2 hub_value(float2 acc, float dg, float mt, float shift, float c0r, float c0i, float2 x) {
     float2 h = make_float2(__fmaf_rn(mt, acc.x, __fmul_rn(dg, x.x)), __fmaf_rn(mt, acc.y, __fmul_rn(dg, x.y)));

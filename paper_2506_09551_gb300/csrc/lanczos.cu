@@ -480,12 +480,12 @@ void ground_state(msb_op* H, double tol, int maxit, const double* start, double*
 // convergent is carried forward: each call folds in levels [k_from, k_to) and
 // keeps the recurrence state per (column, w), so a run of K levels costs O(K)
 // per point instead of O(K^2 / check) for bottom-up re-evaluation at every check.
-// One thread per (active column, w): blockIdx.x the column, blockIdx.y a block of w.  The
+// One thread per (active column, w): blockIdx.y the column, blockIdx.x a block of w.  The
 // levels are a serial chain of two complex reciprocals, so the latency of a division
 // bounds it: one division per reciprocal (cdiv1), and no thread takes a second w.  The
 // column's max |I_new - I_old| and max |I_new| go to diff (zeroed by the caller) by an
 // integer maximum, which orders non-negative doubles.
-// Measured: 24 columns x 400 w, 60 levels 735 -> EVAL_NEW us.
+// Measured: 24 columns x 400 w, 60 levels 735 -> 116 us.
 // ---------------------------------------------------------------------------
 constexpr int kEvalThreads = 64;
 __global__ void __launch_bounds__(kEvalThreads) k_cf_eval(const double* __restrict__ a, const double* __restrict__ b,
@@ -495,9 +495,9 @@ __global__ void __launch_bounds__(kEvalThreads) k_cf_eval(const double* __restri
                                                           int n_w, double eta, double2* __restrict__ gst,
                                                           double2* __restrict__ Cst, double2* __restrict__ Dst, double* I,
                                                           double* diff) {
-    const int c = cols[blockIdx.x];
+    const int c = cols[blockIdx.y];
     const double E0 = E0c[c];
-    const int i = blockIdx.y * kEvalThreads + threadIdx.x;
+    const int i = blockIdx.x * kEvalThreads + threadIdx.x;
     double dmax = 0.0, imax = 0.0;
     if (i < n_w) {
         const double2 one = make_double2(1.0, 0.0);
@@ -1489,7 +1489,7 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
         }
         // Rows shorter than a CTA: no more threads than the row has elements (FP64) or pairs
         // (FP32), in whole warps.  Half of a 256-thread CTA idles on the L = 10 ring's rows of
-        // 126 pairs (160 columns, per level 143 -> F2_NOTE us).  The warps keep their positions,
+        // 126 pairs (160 columns, per level 143 -> 113 us).  The warps keep their positions,
         // so the placement and the hop schedule hold.
         if (maxDdn < 128) fx_threads = int((maxDdn + 31) / 32 * 32);
         if (maxDdn / 2 < kApplyThreads) f2_threads = int(std::max<int64_t>(1, (maxDdn / 2 + 31) / 32) * 32);
@@ -1722,8 +1722,8 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
             {
                 ProfScope ps("cf_eval", st, 0, 40.0 * nact * n_w * double(k - k_eval));
                 MSB_CUDA(cudaMemsetAsync(diff.p, 0, diff.bytes(), st));
-                k_cf_eval<<<dim3(nact, (n_w + kEvalThreads - 1) / kEvalThreads), kEvalThreads, 0, st>>>(a.p, b.p, nv, n0.p, cols.p, k_eval, k, E0d.p, wdev.p, n_w, eta,
-                                                gst.p, Cst.p, Dst.p, I.p, diff.p);
+                k_cf_eval<<<dim3((n_w + kEvalThreads - 1) / kEvalThreads, nact), kEvalThreads, 0, st>>>(
+                    a.p, b.p, nv, n0.p, cols.p, k_eval, k, E0d.p, wdev.p, n_w, eta, gst.p, Cst.p, Dst.p, I.p, diff.p);
                 k_eval = k;
             }
             ++out.launches;

@@ -556,7 +556,7 @@ __global__ void k_block_begin(SeedState* st, ShiftArrays sh, int ns, int nslot) 
 // FP32 (BMAX = 32: the whole window in one pass; NE = 2, the 64 residuals in registers at
 // one CTA per SM): the FP32 pipe and DRAM are about balanced at 256 FMAs per 32 bytes of P
 // and x.  48 shifts, n = 2.9 M, per 32 iterations: 3.4 ms as four windows of 8, 2.5 ms with
-// NE = 1 (bound by the coefficient loads), MEASURED_NE2 with NE = 2.
+// NE = 1 (bound by the coefficient loads), 1.9 ms with NE = 2.
 // FP64 (BMAX = 8, NE = 1): bound by the FP64 pipe (8 FMAs per shift, element and
 // iteration); windows with many shifts go to the tensor cores (flush_tc.cuh), and this
 // kernel returns at once.
@@ -906,16 +906,6 @@ struct SolverImpl {
         grid_mvm = rows.ok ? rows.grid : grid_vec;
         ld = (n + 1) / 2 * 2;
         grid_upd = std::min(grid_for((n * int64_t(sizeof(V)) + 15) / 16, kVecThreads, 3), 3 * sm_count() - 1);
-        if (size_t(W + 1) * ld * sizeof(V) > (size_t(16) << 30)) W = B;
-        try {
-            ring.alloc(size_t(W + 1) * ld);
-        } catch (const Error& e) {
-            if (e.status != MSB_ENOMEM || W == B) throw;
-            cudaGetLastError();
-            W = B;
-            ring.alloc(size_t(W + 1) * ld);
-        }
-        nslot = W + 1;
         p.alloc(n);
         v.alloc(n);
         if (pr.dual) { rt.alloc(n); pt.alloc(n); vt.alloc(n); }
@@ -928,6 +918,25 @@ struct SolverImpl {
         active.alloc(ns); conv.alloc(ns); broken.alloc(ns); nblk.alloc(ns); iters.alloc(ns); zexp.alloc(ns);
         fz_iter.alloc(ns); fz_coef.alloc(ns);
         resid.alloc(ns);
+        shifts_dev.alloc(ns);
+        // The ring comes last, and a long one takes at most 16 GiB and a quarter of the memory
+        // that is left: with less room the window is one block, as small as it can be.
+        const size_t ring_bytes = size_t(W + 1) * ld * sizeof(V);
+        if (ring_bytes > (size_t(16) << 30)) W = B;
+        if (W != B && ring_bytes > (size_t(1) << 30)) {
+            size_t free_b = 0, total_b = 0;
+            MSB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+            if (ring_bytes > free_b / 4) W = B;
+        }
+        try {
+            ring.alloc(size_t(W + 1) * ld);
+        } catch (const Error& e) {
+            if (e.status != MSB_ENOMEM || W == B) throw;
+            cudaGetLastError();
+            W = B;
+            ring.alloc(size_t(W + 1) * ld);
+        }
+        nslot = W + 1;
         tc = std::is_same<V, double2>::value && W == kTcWindow && ns >= kTcMinShifts;
         if (tc) {
             tc_list.alloc(ns); tc_cnt.alloc(1); tc_exp.alloc(2 * ns); tc_mul.alloc(2 * ns);
@@ -936,7 +945,6 @@ struct SolverImpl {
             grid_tc = int(std::min<int64_t>((pr.n_out + kTcCols - 1) / kTcCols, 2 * sm_count()));
             MSB_CUDA(cudaFuncSetAttribute((const void*)k_flush_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmem)));
         }
-        shifts_dev.alloc(ns);
         shifts_dev.upload(pr.shifts.data(), ns, st);
         sh = ShiftArrays{zeta.p, zeta_prev.p, izeta.p, shift.p, coef64.p, (void*)coefv.p,
                          active.p, conv.p, broken.p, nblk.p, iters.p, resid.p, zexp.p, fz_coef.p, fz_iter.p};
