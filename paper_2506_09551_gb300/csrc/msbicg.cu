@@ -22,11 +22,12 @@
 // A shift is frozen when ||r_{m+1}|| / |zeta^k_{m+1}| <= tol ||b|| (Eq. 4).
 //
 // Lagged fused update (the GB300 layout of Eqs. 7-8): the scalars gamma, c
-// of up to `B` consecutive iterations are kept per shift, the seed residuals
-// r_{m0..m0+B-1} are kept in a ring, and one kernel then advances P^k and
-// x^k over those B iterations in registers: one read and one write of each
-// per-shift vector per B iterations instead of per iteration.  The arithmetic
-// and its order are exactly those of the per-iteration update.
+// of a window of W consecutive iterations (64 in FP64, 32 in FP32) are kept per
+// shift, the seed residuals r_{m0..m0+W-1} are kept in a ring, and one kernel then
+// advances P^k and x^k over the window: one read and one write of each per-shift
+// vector per W iterations.  FP32, and FP64 with few shifts: the recurrence in
+// registers, its arithmetic and order exactly those of the per-iteration update.
+// FP64 with more shifts: one contraction on the tensor cores (flush_tc.cuh).
 //
 // Exponent management.  The seed residual of a well-placed seed falls far
 // faster than the residuals of distant shifts (1e-160 after ~1000 iterations
@@ -65,6 +66,9 @@ struct SeedState {
     double2 boa;          // beta_m / alpha_{m-1}
     int f_n, bad_n;       // its rescale exponent; why beta could not be formed
     unsigned cnt_a, cnt_b;   // arrival counters of the two reductions
+    unsigned bar_w, bar_a;   // k_window: arrivals of its workers, and of all its CTAs
+    double2 alpha_w[2];      // k_window: alpha of even and odd iterations, from CTA 0
+    int stop_at;             // k_window: iteration of the window at which the recurrence ended
     double rnorm;         // ||r_m||
     double bnorm;         // ||b||
     double ibnorm;        // 1 / ||b|| (0 for b = 0)
@@ -107,6 +111,30 @@ __device__ __forceinline__ double scale2(double x, int n) {
 }
 __device__ __forceinline__ double2 scale2(double2 v, int n) { return make_double2(scale2(v.x, n), scale2(v.y, n)); }
 
+// alpha_m = rho_m / mu; why it could not be formed, else MSB_OK.
+__device__ __forceinline__ int form_alpha(double2 mu, double2 rho, double2& a) {
+    a = make_double2(0.0, 0.0);
+    if (!cfinite(mu)) return MSB_ENONFINITE;
+    if (mu.x == 0.0 && mu.y == 0.0) return MSB_EBREAKDOWN;
+    a = cdiv1(rho, mu);
+    return cfinite(a) ? MSB_OK : MSB_ENONFINITE;
+}
+
+// beta_{m+1} = rho_{m+1} / rho_m and the exponent f of the rescale, from the sums (rho_{m+1},
+// ||r_{m+1}||^2); why it could not be formed, else MSB_OK.
+__device__ __forceinline__ int form_beta(const double (&v)[3], double2 irho, double ibnorm, double2& b, int& f) {
+    b = make_double2(0.0, 0.0);
+    f = 0;
+    if (!isfinite(v[0]) || !isfinite(v[1]) || !isfinite(v[2])) return MSB_ENONFINITE;
+    if (v[2] == 0.0) return MSB_OK;                         // exact solution: every shift converged
+    if (v[0] == 0.0 && v[1] == 0.0) return MSB_EBREAKDOWN;  // (r, r) = 0 with r != 0
+    b = cmul(make_double2(v[0], v[1]), irho);
+    // bring ||r~|| back near ||b|| once it drifts by more than 2^20
+    const double ratio2 = v[2] * ibnorm * ibnorm;
+    if (ratio2 < 0x1p-40 || ratio2 > 0x1p40) f = -(ilogb(ratio2) >> 1);
+    return MSB_OK;
+}
+
 // First thread block of the product kernel: the iteration's copy of `stop`.
 __device__ __forceinline__ bool mvm_halted(SeedState* st) {
     const int h = st->stop;
@@ -126,15 +154,8 @@ __device__ __forceinline__ void mvm_finish(double (&acc)[2], double* sm, double*
     double mu[2];
     sum_partials_cg<2>(part, gridDim.x, mu, sm);
     if (threadIdx.x == 0) {
-        const double2 m2 = make_double2(mu[0], mu[1]);
-        int bad = MSB_OK;
-        double2 a = make_double2(0.0, 0.0);
-        if (!cfinite(m2)) bad = MSB_ENONFINITE;
-        else if (m2.x == 0.0 && m2.y == 0.0) bad = MSB_EBREAKDOWN;
-        else {
-            a = cdiv1(st->rho, m2);
-            if (!cfinite(a)) bad = MSB_ENONFINITE;
-        }
+        double2 a;
+        const int bad = form_alpha(make_double2(mu[0], mu[1]), st->rho, a);
         if (bad) st->status = bad;
         st->bad = bad;
         st->alpha = a;
@@ -399,23 +420,11 @@ __global__ void __launch_bounds__(kVecThreads, 3) k_seed_update(V* ring, int64_t
     if (!last_cta(&st->cnt_b, gridDim.x - 1)) return;
     sum_partials_cg<3>(part, gridDim.x - 1, acc, sm);
     if (threadIdx.x == 0) {
-        const double2 rho_new = make_double2(acc[0], acc[1]);
-        double2 b = make_double2(0.0, 0.0);
-        int bad = MSB_OK, f = 0;
-        if (!cfinite(rho_new) || !isfinite(acc[2])) {
-            bad = MSB_ENONFINITE;
-        } else if (acc[2] == 0.0) {
-            // exact solution: every shift converged
-        } else if (rho_new.x == 0.0 && rho_new.y == 0.0) {
-            bad = MSB_EBREAKDOWN;                           // (r, r) = 0 with r != 0
-        } else {
-            b = cmul(rho_new, st->irho);
-            // bring ||r~|| back near ||b|| once it drifts by more than 2^20
-            const double ratio2 = acc[2] * st->ibnorm * st->ibnorm;
-            if (ratio2 < 0x1p-40 || ratio2 > 0x1p40) f = -(ilogb(ratio2) >> 1);
-        }
+        double2 b;
+        int f;
+        const int bad = form_beta(acc, st->irho, st->ibnorm, b, f);
         st->beta_n = b;
-        st->rho_n = rho_new;
+        st->rho_n = make_double2(acc[0], acc[1]);
         st->rn2_n = acc[2];
         st->f_n = f;
         st->bad_n = bad;
@@ -454,18 +463,19 @@ __device__ __forceinline__ void shift_scalars_b(SeedState* st, const ShiftArrays
         st->m = m;
         st->j = st->jcur + 1;
         st->rexp[(st->slot0 + st->jcur + 1) % nslot] = rn > 0.0 && isfinite(rn) ? ilogb(rn) + f : 0;
-        // the divisions of the next iteration's scalars, off its critical path
-        const double2 rho = scale2(st->rho_n, 2 * f);
         st->boa = cdiv1(st->beta_n, st->alpha);
-        st->irho = cdiv1(make_double2(1.0, 0.0), rho);
         st->beta = st->beta_n;
-        st->rho = rho;
         st->rnorm = scale2(rn, -st->sexp);
         st->fexp = f;
         st->sexp += f;
         st->nactive = *s_still;
         if (bad) st->status = bad;
         if (bad || *s_still == 0 || m >= st->maxit) st->stop = 1;
+    } else if (threadIdx.x == 32) {
+        // the divisions of the next iteration's scalars: off its critical path, beside each other
+        const double2 rho = scale2(st->rho_n, 2 * f);
+        st->irho = cdiv1(make_double2(1.0, 0.0), rho);
+        st->rho = rho;
     }
 }
 
@@ -541,6 +551,329 @@ __global__ void k_block_begin(SeedState* st, ShiftArrays sh, int ns, int nslot) 
         st->slot0 = (st->slot0 + st->j) % nslot;
         st->m0 = st->m;
         st->j = 0;
+        st->bar_w = 0;
+        st->bar_a = 0;
+        st->stop_at = INT_MAX;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Short vectors: a whole window of iterations in one cooperative launch.
+//
+// With the vectors of an iteration in a few microseconds' reach of the chip, three dependent
+// launches, their fences and the serial scalar work between them decide: 29 us per iteration
+// on the L = 8 ring (n = 3,920), 18 here.  Here the CTAs of one launch keep r, p and v of their elements
+// in registers for the whole window and meet at barriers in global memory (three per
+// iteration): only p (for the gathers of the product, through L2), the residuals for the
+// window's per-shift update and the partial sums leave the SM.  Every worker CTA forms alpha
+// and beta from all partial sums itself.  The per-shift scalars, as long a chain as the vector
+// work, run in a CTA of their own (the last) one iteration behind: after the barrier of
+// iteration j it updates the shifts for j while the workers go on to j + 1.  If the recurrence
+// ended at j, the workers' iteration j + 1 is not counted and nothing reads its vectors.
+//
+// Waits.  A worker arrives at and waits for bar_w after its part of mu and after its p;
+// everybody does at bar_a after the part of rho, the scalar CTA once it has finished the
+// iteration before.  Every worker takes every break from the same sums, or from stop_at < j,
+// which the scalar CTA writes before its arrival for iteration stop_at + 1: all leave at the
+// same iteration.  The launch is cooperative (all CTAs resident) and every wait is bounded.
+// ---------------------------------------------------------------------------
+constexpr int kWaitPolls = 1 << 24;       // about ten seconds
+
+// Loads and stores that other SMs' barrier partners see (L2), never merged or moved by the compiler.
+__device__ __forceinline__ double2 load_l2(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 load_l2(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double load_l2(const double* p) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int load_l2(const int* p) {
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void bar_arrive(unsigned* c) {
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" : : "l"(c) : "memory");
+}
+__device__ __forceinline__ bool bar_wait(const unsigned* c, unsigned target) {
+    for (int i = 0; i < kWaitPolls; ++i) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(c) : "memory");
+        if (v >= target) return true;
+    }
+    return false;
+}
+
+// ((A + c0) x)[s] with x read through L2, four hops in flight; rounded as in the launch-per-product
+// form (hub_value, k_mvm_dot).
+template <typename V>
+__device__ __forceinline__ V gather_ax(const HubView& h, int64_t s, const V* x, V xs, double c0r, double c0i) {
+    using S = scalar_t<V>;
+    const uint32_t iu = uint32_t(s) / uint32_t(h.Ddn), id = uint32_t(s) - iu * uint32_t(h.Ddn);
+    auto hops = [&](V acc, const int32_t* tab, int cnt, int64_t D, int64_t i, int64_t mul, const V* base) {
+        for (int e = 0; e < cnt; e += 4) {
+            int32_t t[4];
+            V v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t[q] = e + q < cnt ? __ldg(tab + int64_t(e + q) * D + i) : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (t[q] >= 0) v[q] = load_l2(base + int64_t(t[q] >> 1) * mul);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (t[q] >= 0) acc = vhop(acc, t[q], v[q]);
+        }
+        return acc;
+    };
+    V acc = hops(vzero(xs), h.hup, __ldg(h.nup + iu), h.Dup, iu, h.Ddn, x + id);
+    acc = hops(acc, h.hdn, __ldg(h.ndn + id), h.Ddn, id, 1, x + int64_t(iu) * h.Ddn);
+    if (h.hup2) {
+        V out = vaxpy(S(-h.t), acc, vscale(h.template diag<S>(iu, id), xs));
+        acc = hops(vzero(xs), h.hup2, __ldg(h.nup2 + iu), h.Dup, iu, h.Ddn, x + id);
+        acc = hops(acc, h.hdn2, __ldg(h.ndn2 + id), h.Ddn, id, 1, x + int64_t(iu) * h.Ddn);
+        out = vaxpy(S(-h.t2), acc, out);
+        return vadd(out, cscale(c0r, c0i, xs));
+    }
+    return hub_value(acc, h.template diag<S>(iu, id), S(-h.t), sizeof(S) == 8 ? S(c0r) : S(0), S(c0r), S(c0i), xs);
+}
+template <typename V>
+__device__ __forceinline__ V gather_ax(const CsrView& m, int64_t s, const V* x, V xs, double c0r, double c0i) {
+    using S = scalar_t<V>;
+    V acc = vzero(xs);
+    const int64_t b = __ldg(m.rowptr + s), e = __ldg(m.rowptr + s + 1);
+    for (int64_t k = b; k < e; k += 4) {
+        V v[4];
+        S a[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (k + q >= e) continue;
+            if constexpr (sizeof(S) == 8) a[q] = __ldg(m.val64 + k + q);
+            else a[q] = __ldg(m.val32 + k + q);
+            v[q] = load_l2(x + __ldg(m.col + k + q));
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (k + q < e) acc = vaxpy(a[q], v[q], acc);
+    }
+    return vadd(acc, cscale(c0r, c0i, xs));
+}
+
+// Sum of the G x NV partial sums of the workers, in a fixed order; every lane of one warp.
+template <int NV>
+__device__ __forceinline__ void window_sum(const double* part, int G, double (&v)[NV]) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = 0.0;
+    for (int b = threadIdx.x & 31; b < G; b += 32) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] += load_l2(part + int64_t(b) * NV + i);
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
+}
+
+// The scalar CTA's loop.
+template <typename V>
+__device__ void window_scalars(SeedState* st, const double* part, int G, const ShiftArrays& sh, int ns, int nslot, int W,
+                               int iters) {
+    __shared__ int s_still, s_end, s_stop;
+    __shared__ double2 s_alpha;
+    for (int j = 0; j < iters; ++j) {
+        if (threadIdx.x < 32) {
+            int end = 0;
+            if (threadIdx.x == 0) {
+                bar_arrive(&st->bar_a);
+                if (!bar_wait(&st->bar_a, unsigned(j + 1) * unsigned(G + 1))) {
+                    st->status = MSB_ETIMEOUT;
+                    end = 1;
+                } else if (const int bad = load_l2(&st->bad)) {
+                    st->status = bad;
+                    end = 1;
+                }
+            }
+            end = __shfl_sync(0xffffffffu, end, 0);
+            double v[3] = {0.0, 0.0, 0.0};
+            if (!end) window_sum<3>(part + (2 + 3 * (j & 1)) * int64_t(G), G, v);
+            if (threadIdx.x == 0) {
+                s_end = end;
+                if (!end) {
+                    double2 b;
+                    int f;
+                    st->bad_n = form_beta(v, st->irho, st->ibnorm, b, f);
+                    st->beta_n = b;
+                    st->rho_n = make_double2(v[0], v[1]);
+                    st->rn2_n = v[2];
+                    st->f_n = f;
+                    st->alpha = s_alpha = load_l2(&st->alpha_w[j & 1]);
+                    st->jcur = st->j;
+                } else {
+                    st->stop = 1;
+                }
+            }
+        }
+        __syncthreads();
+        if (s_end) return;
+        shift_scalars_a<V>(st, s_alpha, sh, ns, W);
+        __syncthreads();
+        shift_scalars_b(st, sh, ns, nslot, &s_still);
+        if (threadIdx.x == 0) {
+            s_stop = st->stop;
+            if (s_stop) {
+                st->stop_at = j;
+                bar_arrive(&st->bar_a);        // for iteration j + 1
+            }
+        }
+        __syncthreads();
+        if (s_stop) return;
+    }
+}
+
+// part: 2 G doubles of mu, then twice 3 G of (rho, ||r||^2), for even and odd iterations.
+template <class View, typename V, int NE>
+__global__ void __launch_bounds__(256, 1) k_window(View op, V* ring, int64_t ld, V* p, int64_t n, double c0r, double c0i,
+                                                   int nslot, SeedState* st, double* part, ShiftArrays sh, int ns, int W,
+                                                   int iters) {
+    if (st->stop) return;                      // set before this launch, or after every CTA has arrived
+    constexpr bool f32 = std::is_same<V, float2>::value;
+    const int G = gridDim.x - 1, b = blockIdx.x;
+    if (b == G) {
+        window_scalars<V>(st, part, G, sh, ns, nslot, W, iters);
+        return;
+    }
+    __shared__ double sm[3 * 256];
+    __shared__ double2 s_c;                    // alpha, then beta
+    __shared__ int s_bad, s_f;
+    const int tid = threadIdx.x;
+    const int64_t nth = int64_t(G) * blockDim.x, t0 = int64_t(b) * blockDim.x + tid;
+    const int slot0 = st->slot0;
+    const double ibnorm = st->ibnorm;
+    double2 rho = st->rho, irho = st->irho;    // used by thread 0 only
+    V r[NE], q[NE], v[NE];
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+        const int64_t s = t0 + i * nth;
+        r[i] = s < n ? ring[int64_t(slot0) * ld + s] : vzero(V{});
+        q[i] = s < n ? p[s] : vzero(V{});
+    }
+    unsigned bars = 0;                         // arrivals of the workers so far
+    for (int j = 0; j < iters; ++j) {
+        if (j > 0) {
+            if (tid == 0) s_bad = bar_wait(&st->bar_w, bars) ? MSB_OK : MSB_ETIMEOUT;
+            __syncthreads();
+            if (s_bad) break;
+        }
+        double acc[2] = {0.0, 0.0};
+        DF4 df;
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+            const int64_t s = t0 + i * nth;
+            if (s >= n) break;
+            v[i] = gather_ax(op, s, p, q[i], c0r, c0i);
+            if constexpr (f32) bil_acc_df(q[i], v[i], df);
+            else bil_acc(q[i], v[i], acc[0], acc[1]);
+        }
+        if constexpr (f32) {
+            acc[0] = df_value(df.rh, df.rl);
+            acc[1] = df_value(df.ih, df.il);
+        }
+        block_sum_sm<2>(acc, sm);
+        bars += G;
+        if (tid < 32) {
+            bool ok = true;
+            if (tid == 0) {
+                part[2 * b] = acc[0];
+                part[2 * b + 1] = acc[1];
+                bar_arrive(&st->bar_w);
+                ok = bar_wait(&st->bar_w, bars);
+            }
+            __syncwarp();
+            double mu[2];
+            window_sum<2>(part, G, mu);
+            if (tid == 0) {
+                double2 a;
+                const int bad = ok ? form_alpha(make_double2(mu[0], mu[1]), rho, a) : int(MSB_ETIMEOUT);
+                s_c = a;
+                s_bad = bad;
+                if (b == 0) {
+                    st->alpha_w[j & 1] = a;
+                    if (bad) st->bad = bad;
+                }
+            }
+        }
+        __syncthreads();
+        const double2 a = s_c;
+        const int bad = s_bad;
+        double sums[3] = {0.0, 0.0, 0.0};
+        if (!bad) {
+            res_sum_t<V> rs;
+            const V af = from_d2<V>(a);
+#pragma unroll
+            for (int i = 0; i < NE; ++i) {
+                if (t0 + i * nth >= n) break;
+                if constexpr (f32) r[i] = axpy_rn(r[i], af, v[i], -1.f);
+                else r[i] = cfma(make_double2(-a.x, -a.y), v[i], r[i]);
+                rs.add(r[i]);
+            }
+            rs.get(sums);
+            block_sum_sm<3>(sums, sm);
+        }
+        if (tid < 32) {
+            double* pr = part + (2 + 3 * (j & 1)) * int64_t(G);
+            bool ok = true;
+            if (tid == 0) {
+                if (!bad) {
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) pr[3 * int64_t(b) + i] = sums[i];
+                }
+                bar_arrive(&st->bar_a);
+                ok = bad || bar_wait(&st->bar_a, unsigned(j + 1) * unsigned(G + 1));
+            }
+            __syncwarp();
+            if (!bad) window_sum<3>(pr, G, sums);
+            if (tid == 0) {
+                double2 bt = make_double2(0.0, 0.0);
+                int f = 0, e = bad;
+                if (!e) e = !ok ? int(MSB_ETIMEOUT) : load_l2(&st->stop_at) < j ? int(MSB_EMAXITER) : form_beta(sums, irho, ibnorm, bt, f);
+                s_c = bt;
+                s_f = f;
+                s_bad = e;
+            }
+        }
+        __syncthreads();
+        if (s_bad) break;                      // the same in every worker
+        const double2 beta = s_c;
+        const int f = s_f;
+        V* __restrict__ rn = ring + int64_t((slot0 + j + 1) % nslot) * ld;
+        const V bv = from_d2<V>(beta);
+        const double sc = scale2(1.0, f);
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+            const int64_t s = t0 + i * nth;
+            if (s >= n) break;
+            if constexpr (f32) q[i] = axpy_rn(r[i], bv, q[i], 1.f);
+            else q[i] = cfma(bv, q[i], r[i]);
+            if (f != 0) {
+                q[i] = cscale(sc, 0.0, q[i]);
+                r[i] = cscale(sc, 0.0, r[i]);
+            }
+            rn[s] = r[i];
+            p[s] = q[i];
+        }
+        __syncthreads();
+        bars += G;
+        if (tid == 0 && j + 1 < iters) {
+            bar_arrive(&st->bar_w);
+            rho = scale2(make_double2(sums[0], sums[1]), 2 * f);
+            irho = cdiv1(make_double2(1.0, 0.0), rho);
+        }
     }
 }
 
@@ -761,6 +1094,9 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         st->bad_n = 0;
         st->cnt_a = 0;
         st->cnt_b = 0;
+        st->bar_w = 0;
+        st->bar_a = 0;
+        st->stop_at = INT_MAX;
         st->stop = (bn == 0.0 || maxit <= 0) ? 1 : 0;
         if (bn != 0.0 && st->rho.x == 0.0 && st->rho.y == 0.0) { st->status = MSB_EBREAKDOWN; st->stop = 1; }
         st->nactive = bn == 0.0 ? 0 : ns;
@@ -861,6 +1197,50 @@ struct SolverImpl {
         }
     }
 
+    // A whole window of iterations in one launch (k_window), on the shape of coop_plan.
+    int coop_t = 0, coop_ne = 0, coop_g = 0;
+    template <class View>
+    void window(const View& view) {
+        if constexpr (!std::is_same<View, SumView>::value) {
+            ProfScope ps("seed_window", st, 0, 0);
+            auto go = [&](auto kern) {
+                View vw = view;
+                V *rg = ring.p, *pp = p.p;
+                int64_t l = ld, n = pr.n;
+                double cr = pr.c0.x, ci = pr.c0.y;
+                int sl = nslot, ns = pr.ns, w = W;
+                SeedState* s = state.p;
+                double* pa = part.p;
+                void* args[] = {&vw, &rg, &l, &pp, &n, &cr, &ci, &sl, &s, &pa, &sh, &ns, &w, &w};
+                MSB_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(coop_g + 1), dim3(coop_t), args, 0, st));
+            };
+            if (coop_ne == 1) go(k_window<View, V, 1>);
+            else go(k_window<View, V, 2>);
+        }
+    }
+
+    // Launch shape of k_window, or none (coop_g = 0): up to 384 elements per worker (n = 57,984
+    // on 152 SMs), the smallest CTAs that take one element per thread (the FP64 pipe of an SM
+    // issues one warp at a time) and have a thread per shift.  Measured, us per iteration, graph of
+    // launches -> k_window.  FP64: Hubbard sectors n = 36, 3,920, 15,876 and 52,920 with 41 shifts
+    // 42 -> 28, 29.4 -> 17.9, 29.9 -> 20.2, 38.6 -> 32.2; random matrices n = 38,000 35.7 -> 25.3,
+    // 60,001 40.1 -> 39.8, 100,003 (four elements per thread) 49 -> 85.  FP32: 28.5 -> 17.5 at
+    // n = 3,920, 29.3 -> 23.6 at 52,920.
+    void coop_plan(bool view_ok) {
+        if (pr.dual || !view_ok) return;
+        int dev = 0, ok = 0;
+        MSB_CUDA(cudaGetDevice(&dev));
+        MSB_CUDA(cudaDeviceGetAttribute(&ok, cudaDevAttrCooperativeLaunch, dev));
+        const int most = sm_count() - 1;                          // one CTA per SM, one of them for the scalars
+        if (!ok || most < 1) return;
+        int t = 64;
+        while (t < 256 && (pr.n > int64_t(t) * most || pr.ns > t)) t *= 2;
+        if (pr.n > int64_t(384) * most) return;
+        coop_ne = pr.n <= int64_t(t) * most ? 1 : 2;
+        coop_t = t;
+        coop_g = int((pr.n + int64_t(t) * coop_ne - 1) / (int64_t(t) * coop_ne));
+    }
+
     // End of a window: the per-shift update of its iterations, then an empty window.
     void flush() {
         {
@@ -904,13 +1284,14 @@ struct SolverImpl {
         rows = op->kind == 2 ? (f32 ? op->plan32 : op->plan64) : row_plan<V>(op, 1);
         if (op->kind == 2) rparts = f32 ? op->parts32.p : op->parts64.p;
         grid_mvm = rows.ok ? rows.grid : grid_vec;
+        coop_plan(!std::is_same<View, SumView>::value);
         ld = (n + 1) / 2 * 2;
         grid_upd = std::min(grid_for((n * int64_t(sizeof(V)) + 15) / 16, kVecThreads, 3), 3 * sm_count() - 1);
         p.alloc(n);
         v.alloc(n);
         if (pr.dual) { rt.alloc(n); pt.alloc(n); vt.alloc(n); }
         Pbuf.alloc(size_t(ns) * pr.n_out);
-        part.alloc(size_t(std::max(std::max(grid_vec, grid_mvm), grid_upd)) * 4);
+        part.alloc(std::max(size_t(std::max(std::max(grid_vec, grid_mvm), grid_upd)) * 4, size_t(coop_g) * 8));
         state.alloc(1);
         zeta.alloc(ns); zeta_prev.alloc(ns); izeta.alloc(ns); shift.alloc(ns);
         coef64.alloc(size_t(ns) * W * 2);
@@ -960,8 +1341,10 @@ struct SolverImpl {
         }
         launches += 2;
         MSB_LAUNCH_CHECK();
-        const int64_t per_block = (pr.dual ? 4 : 3) * int64_t(B);       // kernels per block of iterations
-        const int64_t max_blocks = (int64_t(pr.maxit) + B - 1) / B + 1;
+        const bool coop = coop_g > 0;
+        const int BB = coop ? W : B;                                    // iterations per launch of a block
+        const int64_t per_block = coop ? 1 : (pr.dual ? 4 : 3) * int64_t(B);   // kernels per block
+        const int64_t max_blocks = (int64_t(pr.maxit) + BB - 1) / BB + 1;
         int64_t blocks = 0;
         if (prof_on()) {
             // Profiled: direct launches, one sync per block, and one after each fused
@@ -972,12 +1355,17 @@ struct SolverImpl {
                 MSB_CUDA(cudaStreamSynchronize(st));
             };
             for (;;) {
-                for (int i = 0; i < B; ++i) iteration(view);
+                if (coop) window(view);
+                else
+                    for (int i = 0; i < B; ++i) iteration(view);
                 launches += per_block;
                 ++blocks;
                 look();
+                if (coop)
+                    prof_patch_last("seed_window", hs.j * (8.0 * n * csz + op->matrix_bytes(csz)),
+                                    hs.j * (op->hx_flops() + 44.0 * n));
                 const bool end = hs.stop || blocks > max_blocks + 2;
-                if (end || blocks * B % W == 0) {
+                if (end || blocks * BB % W == 0) {
                     flush();
                     look();
                     const double no = double(pr.n_out) * csz;
@@ -988,16 +1376,17 @@ struct SolverImpl {
                 if (end) break;
             }
             prof_collect();
-            out.flushes = blocks;
         } else {
 
-        // One block of B iterations, captured once.
+        // One block of B iterations, captured once (k_window: launched directly).
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
-        MSB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        for (int i = 0; i < B; ++i) iteration(view);
-        MSB_CUDA(cudaStreamEndCapture(st, &graph));
-        MSB_CUDA(cudaGraphInstantiate(&exec, graph, 0));
+        if (!coop) {
+            MSB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+            for (int i = 0; i < B; ++i) iteration(view);
+            MSB_CUDA(cudaStreamEndCapture(st, &graph));
+            MSB_CUDA(cudaGraphInstantiate(&exec, graph, 0));
+        }
 
         HostBuf<SeedState> hstate(2);
         cudaEvent_t ev[2];
@@ -1007,9 +1396,10 @@ struct SolverImpl {
         // Two blocks in flight: launch block i, then look at the state copied
         // after block i-1.  Blocks launched after convergence return at once.
         while (!finished) {
-            MSB_CUDA(cudaGraphLaunch(exec, st));
+            if (coop) window(view);
+            else MSB_CUDA(cudaGraphLaunch(exec, st));
             launches += per_block;
-            if ((blocks + 1) * B % W == 0) { flush(); window_begin(); }
+            if ((blocks + 1) * BB % W == 0) { flush(); window_begin(); }
             const int slot = int(blocks & 1);
             MSB_CUDA(cudaMemcpyAsync(&hstate.p[slot], state.p, sizeof(SeedState), cudaMemcpyDeviceToHost, st));
             MSB_CUDA(cudaEventRecord(ev[slot], st));
@@ -1025,10 +1415,10 @@ struct SolverImpl {
         MSB_CUDA(cudaStreamSynchronize(st));
         cudaEventDestroy(ev[0]);
         cudaEventDestroy(ev[1]);
-        cudaGraphExecDestroy(exec);
-        cudaGraphDestroy(graph);
-        out.flushes = blocks;
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
         }
+        out.flushes = blocks * (BB / B);
 
         SeedState fs;
         MSB_CUDA(cudaMemcpyAsync(&fs, state.p, sizeof(SeedState), cudaMemcpyDeviceToHost, st));
