@@ -1577,10 +1577,9 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
     // L1/shared pipe) overlaps the orth pass of the other (bound by DRAM).  Each group's
     // levels are ordered on its own stream; the groups meet at every convergence check.
     // With the profiler on, one group, so that every launch is timed alone.
-    // Small batches take one group: a level is then two launches long, not bound by the
-    // pipes, and a second stream only doubles the launches (map of the L = 8 ring, 41
-    // columns of 4,900: MAPL8_NOTE).
-    const int ngrp = prof_on() || all_elems < 4e6 ? 1 : 2;
+    // Small batches gain as well (one group -> two: map of the L = 8 ring, 41 columns of 4,900,
+    // 70.1 -> 66.2 ms; 60 levels of 16 and 40 columns of 63,504, 4.44 -> 3.89 and 8.70 -> 7.67 ms).
+    const int ngrp = prof_on() ? 1 : 2;
     // a column's sums close in its own last CTA where the CTAs per column are few
     const bool tails = cpc != 2 && nblkA <= 512;
     cudaStream_t gs[2] = {st, nullptr};
