@@ -1578,7 +1578,7 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
     // levels are ordered on its own stream; the groups meet at every convergence check.
     // With the profiler on, one group, so that every launch is timed alone.
     // Small batches gain as well (one group -> two: map of the L = 8 ring, 41 columns of 4,900,
-    // 70.1 -> 66.2 ms; 60 levels of 16 and 40 columns of 63,504, 4.44 -> 3.89 and 8.70 -> 7.67 ms).
+    // 70.1 -> 65.7 ms; 60 levels of 16 and 40 columns of 63,504, 4.44 -> 3.89 and 8.70 -> 7.65 ms).
     const int ngrp = prof_on() ? 1 : 2;
     // a column's sums close in its own last CTA where the CTAs per column are few
     const bool tails = cpc != 2 && nblkA <= 512;
