@@ -295,7 +295,7 @@ msb_status msb_ground_state_noalloc(msb_op *H, double tol, int maxit, const doub
  * frozen once ||r_m|| / |zeta_m^(k)| <= tol ||b||.  Optional HOST outputs
  * (may be NULL): iters[k], resid[k] (that ratio / ||b|| at freeze), converged[k].
  * `block` (1..16, 0 = auto): iterations per launched graph, after which convergence is
- * looked at.  The vectors p^(k), x^(k) are advanced once per window of 64 (FP64) or 32
+ * looked at.  The vectors p^(k), x^(k) are advanced once per window of 56 (FP64) or 32
  * (FP32) iterations from the stored seed residuals, or once per `block` when memory is
  * short, with coefficients from the same recurrences.
  * Returns MSB_EMAXITER (results still written) if a shift did not converge

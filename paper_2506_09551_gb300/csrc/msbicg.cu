@@ -22,7 +22,7 @@
 // A shift is frozen when ||r_{m+1}|| / |zeta^k_{m+1}| <= tol ||b|| (Eq. 4).
 //
 // Lagged fused update (the GB300 layout of Eqs. 7-8): the scalars gamma, c
-// of a window of W consecutive iterations (64 in FP64, 32 in FP32) are kept per
+// of a window of W consecutive iterations (56 in FP64, 32 in FP32) are kept per
 // shift, the seed residuals r_{m0..m0+W-1} are kept in a ring, and one kernel then
 // advances P^k and x^k over the window: one read and one write of each per-shift
 // vector per W iterations.  FP32, and FP64 with few shifts: the recurrence in
@@ -1138,7 +1138,7 @@ struct SolverImpl {
     const SolveProblem& pr;
     cudaStream_t st;
     int nslot, B, grid_vec, grid_flush, grid_mvm, grid_upd;
-    // Window of the per-shift update: 32 iterations in FP32, 64 in FP64 (one contraction on
+    // Window of the per-shift update: 32 iterations in FP32, 56 in FP64 (one contraction on
     // the tensor cores), whatever the block B of iterations per graph; B when the ring of
     // residuals would take too much memory.
     int W = 0, grid_tc = 0;
@@ -1277,7 +1277,7 @@ struct SolverImpl {
         op = op_;
         const int64_t n = pr.n, ns = pr.ns;
         B = pr.block;
-        W = std::is_same<V, float2>::value ? 32 : kTcWindow;
+        W = std::is_same<V, float2>::value ? 32 : kTcWindow / B * B;    // whole blocks
         grid_vec = grid_for(n, 256, 8);
         grid_flush = std::is_same<V, float2>::value ? grid_for((pr.n_out + 1) / 2, 256, 4) : grid_for(pr.n_out, 256, 8);
         constexpr bool f32 = std::is_same<V, float2>::value;
@@ -1318,11 +1318,11 @@ struct SolverImpl {
             ring.alloc(size_t(W + 1) * ld);
         }
         nslot = W + 1;
-        tc = std::is_same<V, double2>::value && W == kTcWindow && ns >= kTcMinShifts;
+        tc = std::is_same<V, double2>::value && W == kTcWindow / B * B && ns >= kTcMinShifts;
         if (tc) {
             tc_list.alloc(ns); tc_cnt.alloc(1); tc_exp.alloc(2 * ns); tc_mul.alloc(2 * ns);
             tc_frag.alloc(size_t((ns + 3) / 4) * kTcSteps * kTcDigits * 32);
-            tcc = TcCoef{tc_list.p, tc_cnt.p, tc_mul.p, tc_exp.p, tc_frag.p, state.p->rexp};
+            tcc = TcCoef{tc_list.p, tc_cnt.p, tc_mul.p, tc_exp.p, tc_frag.p, coef64.p, nblk.p, W, state.p->rexp};
             grid_tc = int(std::min<int64_t>((pr.n_out + kTcCols - 1) / kTcCols, 2 * sm_count()));
             MSB_CUDA(cudaFuncSetAttribute((const void*)k_flush_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmem)));
         }
