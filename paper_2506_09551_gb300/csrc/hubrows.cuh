@@ -307,7 +307,9 @@ template <typename V, class Epi>
 void launch_hub_rows(const RowPlan& p, const HubPart* dparts, const V* x, int64_t ldx, int nvec, double c0r, Epi epi,
                      cudaStream_t st) {
     auto go = [&](auto kern) {
-        if (p.smem > 48 * 1024)
+        // dynamic and static shared memory (4 KB of an epilogue's block sum) together count
+        // against the 48 KB that a launch gets without asking
+        if (p.smem > 40 * 1024)
             MSB_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(p.smem)));
         kern<<<dim3(p.grid, nvec), p.threads, p.smem, st>>>(p.one, dparts, p.np, x, ldx, p.tiles, c0r, 1.0, epi);
     };
