@@ -251,6 +251,8 @@ __device__ __forceinline__ float2 hub_value(float2 acc, float dg, float mt, floa
     return make_float2(__fadd_rn(h.x, c.x), __fadd_rn(h.y, c.y));
 }
 
+constexpr size_t kMaxRowBytes = 112 * 1024;      // two CTAs per SM
+
 // Tiles of an operator's blocks and the launch shape for vectors of element V with
 // `nvec` columns; ok = false: the element-wise kernels (a second hopping amplitude,
 // Peierls phases, rows too long for shared memory).
@@ -297,7 +299,7 @@ RowPlan row_plan(const msb_op* op, int nvec) {
     p.one = p.parts[0];
     const int64_t most = 4096;
     p.grid = int(t0 <= most ? t0 : (t0 + (t0 + most - 1) / most - 1) / ((t0 + most - 1) / most));
-    p.ok = p.smem <= 112 * 1024 && t0 < (int64_t(1) << 31);
+    p.ok = p.smem <= kMaxRowBytes && t0 < (int64_t(1) << 31);
     return p;
 }
 
@@ -309,8 +311,7 @@ void launch_hub_rows(const RowPlan& p, const HubPart* dparts, const V* x, int64_
     auto go = [&](auto kern) {
         // dynamic and static shared memory (4 KB of an epilogue's block sum) together count
         // against the 48 KB that a launch gets without asking
-        if (p.smem > 40 * 1024)
-            MSB_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(p.smem)));
+        if (p.smem > 40 * 1024) raise_shared_limit((const void*)kern, kMaxRowBytes);
         kern<<<dim3(p.grid, nvec), p.threads, p.smem, st>>>(p.one, dparts, p.np, x, ldx, p.tiles, c0r, 1.0, epi);
     };
     if constexpr (std::is_same<V, float2>::value) {

@@ -201,6 +201,12 @@ __device__ __forceinline__ double2 cdiv1(double2 a, double2 b) {
     return make_double2(fma(a.x, bx, a.y * by) * r, fma(a.y, bx, -a.x * by) * r);
 }
 
+// Raise a kernel's limit of dynamic shared memory.  The limit belongs to the process: callers pass
+// the same value for a kernel every time, so that no thread lowers it under another's launch.
+inline void raise_shared_limit(const void* kern, size_t bytes) {
+    MSB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
+}
+
 // CUDA device sanity check used by every compute entry point.
 void require_device();
 msb_status guard(const char* fn, const std::function<void()>& body);

@@ -609,6 +609,7 @@ __device__ __forceinline__ void cf_tail(const CFTail& t, const double* part, int
     }
 }
 
+constexpr int64_t kMaxCfRowBytes = 200 * 1024;   // staged rows of a CTA
 constexpr int kMaxHops = 32;     // up-spin hops per row (a 2D 3 x 4 cluster has 24 bonds)
 
 // Pass A for the Hubbard operator, one CTA per (row u, active column): row u
@@ -1477,7 +1478,7 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
         // the FP32 two-element kernels, padded to 16 bytes), diagonal table
         const int zw = pair ? kRowZeroWords : 2;
         hub_smem = (maxDdn + zw) * int64_t(sizeof(C)) + 3 * (maxL + 1) * 8;
-        rows = rows && hub_smem <= 160 * 1024;
+        rows = rows && hub_smem <= 160 * 1024;       // two columns per CTA: up to kMaxCfRowBytes
         // FP64 fixed-point kernel: rows of up to 1024 elements take 128-thread CTAs (~7
         // elements per thread at L = 12, so the staging barrier and the block reduction
         // are paid over twice the work); longer rows keep 256 threads, where shared
@@ -1512,7 +1513,7 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
             else if (pair && cpc == 2) {
                 fn = sgn ? (const void*)k_cf_apply_hub_f2x2c2<true> : (const void*)k_cf_apply_hub_f2x2c2<false>;
                 hub_smem = 2 * (maxDdn + zw) * int64_t(sizeof(C)) + 2 * 3 * (maxL + 1) * 4;
-                if (hub_smem > 200 * 1024) {               // rows too long for two per CTA
+                if (hub_smem > kMaxCfRowBytes) {             // rows too long for two per CTA
                     cpc = 1;
                     hub_smem = (maxDdn + zw) * int64_t(sizeof(C)) + 3 * (maxL + 1) * 8;
                     fn = sgn ? (const void*)k_cf_apply_hub_f2x2<false, true, 6> : (const void*)k_cf_apply_hub_f2x2<false, false, 6>;
@@ -1527,7 +1528,7 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
                            : (sgn ? (const void*)k_cf_apply_hub_f2x2<false, true, 6> : (const void*)k_cf_apply_hub_f2x2<false, false, 6>);
             else
                 fn = multi ? (const void*)k_cf_apply_hub<float2, true> : (const void*)k_cf_apply_hub<float2, false>;
-            MSB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(hub_smem)));
+            raise_shared_limit(fn, kMaxCfRowBytes);
             if (cpc == 3)      // eight rows of shared memory per SM: take the largest carve-out
                 MSB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
                                               int(cudaSharedmemCarveoutMaxShared)));

@@ -1324,7 +1324,7 @@ struct SolverImpl {
             tc_frag.alloc(size_t((ns + 3) / 4) * kTcSteps * kTcDigits * 32);
             tcc = TcCoef{tc_list.p, tc_cnt.p, tc_mul.p, tc_exp.p, tc_frag.p, coef64.p, nblk.p, W, state.p->rexp};
             grid_tc = int(std::min<int64_t>((pr.n_out + kTcCols - 1) / kTcCols, 2 * sm_count()));
-            MSB_CUDA(cudaFuncSetAttribute((const void*)k_flush_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTcSmem)));
+            raise_shared_limit((const void*)k_flush_tc, kTcSmem);
         }
         shifts_dev.upload(pr.shifts.data(), ns, st);
         sh = ShiftArrays{zeta.p, zeta_prev.p, izeta.p, shift.p, coef64.p, (void*)coefv.p,
