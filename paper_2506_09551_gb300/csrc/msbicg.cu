@@ -848,10 +848,19 @@ __global__ void __launch_bounds__(256, 1) k_window(View op, V* ring, int64_t ld,
             }
         }
         __syncthreads();
-        if (s_bad) break;                      // the same in every worker
+        const int end = s_bad;                 // the same in every worker
+        V* __restrict__ rn = ring + int64_t((slot0 + j + 1) % nslot) * ld;
+        if (end) {
+            // beta could not be formed: the iteration counts, and k_rrec reads its residual
+            if (!bad && (end == MSB_EBREAKDOWN || end == MSB_ENONFINITE)) {
+#pragma unroll
+                for (int i = 0; i < NE; ++i)
+                    if (t0 + i * nth < n) rn[t0 + i * nth] = r[i];
+            }
+            break;
+        }
         const double2 beta = s_c;
         const int f = s_f;
-        V* __restrict__ rn = ring + int64_t((slot0 + j + 1) % nslot) * ld;
         const V bv = from_d2<V>(beta);
         const double sc = scale2(1.0, f);
 #pragma unroll
