@@ -1285,8 +1285,11 @@ struct SolverImpl {
     void run(const msb_op* op_, const View& view, SolveResult& out) {
         op = op_;
         const int64_t n = pr.n, ns = pr.ns;
-        B = pr.block;
-        W = std::is_same<V, float2>::value ? 32 : kTcWindow / B * B;    // whole blocks
+        // A window is whole blocks, and the same for every block the caller asks for (bitwise equal
+        // results): FP64 graphs hold at most 8 iterations.
+        static_assert(kTcWindow % 8 == 0, "whole blocks per window");
+        B = std::min(pr.block, std::is_same<V, float2>::value ? 16 : 8);
+        W = std::is_same<V, float2>::value ? 32 : kTcWindow;
         grid_vec = grid_for(n, 256, 8);
         grid_flush = std::is_same<V, float2>::value ? grid_for((pr.n_out + 1) / 2, 256, 4) : grid_for(pr.n_out, 256, 8);
         constexpr bool f32 = std::is_same<V, float2>::value;
@@ -1327,7 +1330,7 @@ struct SolverImpl {
             ring.alloc(size_t(W + 1) * ld);
         }
         nslot = W + 1;
-        tc = std::is_same<V, double2>::value && W == kTcWindow / B * B && ns >= kTcMinShifts;
+        tc = std::is_same<V, double2>::value && W == kTcWindow && ns >= kTcMinShifts;
         if (tc) {
             tc_list.alloc(ns); tc_cnt.alloc(1); tc_exp.alloc(2 * ns); tc_mul.alloc(2 * ns);
             tc_frag.alloc(size_t((ns + 3) / 4) * kTcSteps * kTcDigits * 32);
