@@ -292,28 +292,31 @@ __device__ __forceinline__ void shift_scalars_a(SeedState* st, double2 alpha, co
     }
 }
 
-// Sums of one residual element: x.x, y.y and x.y of its parts, from which rho =
-// (Sxx - Syy) + 2 i Sxy and ||r||^2 = Sxx + Syy follow: three products per element
-// where rho and the norm separately take six.
+// Sums over residual elements: rho = sum (x.x - y.y) + 2 i sum x.y and ||r||^2 = Re rho + 2 sum y.y,
+// four products per element where rho and the norm separately take six.  Re rho is summed term by
+// term: a difference of sum x.x and sum y.y would be rounded at the size of ||r||^2, which loses
+// rho when the residual is close to isotropic.
 struct ResSum {
-    double xx = 0.0, yy = 0.0, xy = 0.0;
+    double re = 0.0, yy = 0.0, xy = 0.0;
     __device__ __forceinline__ void add(double2 r) {
-        xx = fma(r.x, r.x, xx);
+        re = fma(r.x, r.x, fma(-r.y, r.y, re));
         yy = fma(r.y, r.y, yy);
         xy = fma(r.x, r.y, xy);
     }
-    __device__ __forceinline__ void get(double (&a)[3]) const { a[0] = xx - yy; a[1] = 2.0 * xy; a[2] = xx + yy; }
+    __device__ __forceinline__ void get(double (&a)[3]) const { a[0] = re; a[1] = 2.0 * xy; a[2] = fma(2.0, yy, re); }
 };
 struct ResSumF {
-    float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f, ch = 0.f, cl = 0.f;
+    float rh = 0.f, rl = 0.f, yh = 0.f, yl = 0.f, ch = 0.f, cl = 0.f;
     __device__ __forceinline__ void add(float2 r) {
-        df_add_prod(xh, xl, r.x, r.x);
+        df_add_prod(rh, rl, r.x, r.x);
+        df_add_prod(rh, rl, -r.y, r.y);
         df_add_prod(yh, yl, r.y, r.y);
         df_add_prod(ch, cl, r.x, r.y);
     }
     __device__ __forceinline__ void get(double (&a)[3]) const {
-        const double xx = df_value(xh, xl), yy = df_value(yh, yl);
-        a[0] = xx - yy; a[1] = 2.0 * df_value(ch, cl); a[2] = xx + yy;
+        a[0] = df_value(rh, rl);
+        a[1] = 2.0 * df_value(ch, cl);
+        a[2] = fma(2.0, df_value(yh, yl), a[0]);
     }
 };
 template <typename V> using res_sum_t = typename std::conditional<std::is_same<V, float2>::value, ResSumF, ResSum>::type;
