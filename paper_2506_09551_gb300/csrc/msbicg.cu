@@ -62,7 +62,7 @@ struct SeedState {
     double2 beta;         // beta_m: built p_m (0 at m = 0)
     double2 beta_n, rho_n;   // beta_{m+1}, (r~_{m+1}, r~_{m+1}) before the rescale
     double rn2_n;         // ||r~_{m+1}||^2
-    double2 irho;         // 1 / rho_m
+    double2 irho;         // 1 / rho_m (not finite if that is not representable)
     double2 boa;          // beta_m / alpha_{m-1}
     int f_n, bad_n;       // its rescale exponent; why beta could not be formed
     unsigned cnt_a, cnt_b;   // arrival counters of the two reductions
@@ -121,14 +121,16 @@ __device__ __forceinline__ int form_alpha(double2 mu, double2 rho, double2& a) {
 }
 
 // beta_{m+1} = rho_{m+1} / rho_m and the exponent f of the rescale, from the sums (rho_{m+1},
-// ||r_{m+1}||^2); why it could not be formed, else MSB_OK.
-__device__ __forceinline__ int form_beta(const double (&v)[3], double2 irho, double ibnorm, double2& b, int& f) {
+// ||r_{m+1}||^2); why it could not be formed, else MSB_OK.  irho = 1 / rho_m was formed beside the
+// vectors, off the chain (a division here: 2% of the L = 8 solve).
+__device__ __forceinline__ int form_beta(const double (&v)[3], double2 rho, double2 irho, double ibnorm, double2& b, int& f) {
     b = make_double2(0.0, 0.0);
     f = 0;
     if (!isfinite(v[0]) || !isfinite(v[1]) || !isfinite(v[2])) return MSB_ENONFINITE;
     if (v[2] == 0.0) return MSB_OK;                         // exact solution: every shift converged
     if (v[0] == 0.0 && v[1] == 0.0) return MSB_EBREAKDOWN;  // (r, r) = 0 with r != 0
     b = cmul(make_double2(v[0], v[1]), irho);
+    if (!cfinite(irho)) b = cdiv1(make_double2(v[0], v[1]), rho);       // rho_m is subnormal
     // bring ||r~|| back near ||b|| once it drifts by more than 2^20
     const double ratio2 = v[2] * ibnorm * ibnorm;
     if (ratio2 < 0x1p-40 || ratio2 > 0x1p40) f = -(ilogb(ratio2) >> 1);
@@ -425,7 +427,7 @@ __global__ void __launch_bounds__(kVecThreads, 3) k_seed_update(V* ring, int64_t
     if (threadIdx.x == 0) {
         double2 b;
         int f;
-        const int bad = form_beta(acc, st->irho, st->ibnorm, b, f);
+        const int bad = form_beta(acc, st->rho, st->irho, st->ibnorm, b, f);
         st->beta_n = b;
         st->rho_n = make_double2(acc[0], acc[1]);
         st->rn2_n = acc[2];
@@ -710,7 +712,7 @@ __device__ void window_scalars(SeedState* st, const double* part, int G, const S
                 if (!end) {
                     double2 b;
                     int f;
-                    st->bad_n = form_beta(v, st->irho, st->ibnorm, b, f);
+                    st->bad_n = form_beta(v, st->rho, st->irho, st->ibnorm, b, f);
                     st->beta_n = b;
                     st->rho_n = make_double2(v[0], v[1]);
                     st->rn2_n = v[2];
@@ -844,7 +846,7 @@ __global__ void __launch_bounds__(256, 1) k_window(View op, V* ring, int64_t ld,
             if (tid == 0) {
                 double2 bt = make_double2(0.0, 0.0);
                 int f = 0, e = bad;
-                if (!e) e = !ok ? int(MSB_ETIMEOUT) : load_l2(&st->stop_at) < j ? int(MSB_EMAXITER) : form_beta(sums, irho, ibnorm, bt, f);
+                if (!e) e = !ok ? int(MSB_ETIMEOUT) : load_l2(&st->stop_at) < j ? int(MSB_EMAXITER) : form_beta(sums, rho, irho, ibnorm, bt, f);
                 s_c = bt;
                 s_f = f;
                 s_bad = e;
