@@ -1146,6 +1146,17 @@ __global__ void k_zero(V* x, int64_t n) {
 // ---------------------------------------------------------------------------
 // Host driver
 // ---------------------------------------------------------------------------
+thread_local SolverLimits g_solver_limits;
+
+struct GraphOwner {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    ~GraphOwner() {
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
+    }
+};
+
 template <typename V>
 struct SolverImpl {
     using C = V;
@@ -1211,11 +1222,15 @@ struct SolverImpl {
         }
     }
 
-    // A whole window of iterations in one launch (k_window), on the shape of coop_plan.
+    // A whole window of iterations in one launch (k_window), on the shape of coop_plan.  False: the
+    // runtime refused it, since its CTAs do not fit the SMs at once (a context limited to part of
+    // the SMs); nothing ran.
     int coop_t = 0, coop_ne = 0, coop_g = 0;
     template <class View>
-    void window(const View& view) {
+    bool window(const View& view) {
+        cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
         if constexpr (!std::is_same<View, SumView>::value) {
+            if (g_solver_limits.refuse_cooperative) return false;
             ProfScope ps("seed_window", st, 0, 0);
             auto go = [&](auto kern) {
                 View vw = view;
@@ -1226,11 +1241,17 @@ struct SolverImpl {
                 SeedState* s = state.p;
                 double* pa = part.p;
                 void* args[] = {&vw, &rg, &l, &pp, &n, &cr, &ci, &sl, &s, &pa, &sh, &ns, &w, &w};
-                MSB_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(coop_g + 1), dim3(coop_t), args, 0, st));
+                e = cudaLaunchCooperativeKernel((const void*)kern, dim3(coop_g + 1), dim3(coop_t), args, 0, st);
             };
             if (coop_ne == 1) go(k_window<View, V, 1>);
             else go(k_window<View, V, 2>);
         }
+        if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) {
+            MSB_CUDA(e);
+            return true;
+        }
+        cudaGetLastError();
+        return false;
     }
 
     // Launch shape of k_window, or none (coop_g = 0): up to 384 elements per worker (n = 57,984
@@ -1358,11 +1379,35 @@ struct SolverImpl {
         }
         launches += 2;
         MSB_LAUNCH_CHECK();
-        const bool coop = coop_g > 0;
-        const int BB = coop ? W : B;                                    // iterations per launch of a block
-        const int64_t per_block = coop ? 1 : (pr.dual ? 4 : 3) * int64_t(B);   // kernels per block
-        const int64_t max_blocks = (int64_t(pr.maxit) + BB - 1) / BB + 1;
-        int64_t blocks = 0;
+        bool coop = false;
+        int BB = 0;                                 // iterations per launch of a block
+        int64_t per_block = 0, max_blocks = 0, blocks = 0;      // kernels per block
+        auto form = [&](bool cooperative) {
+            coop = cooperative;
+            BB = coop ? W : B;
+            per_block = coop ? 1 : (pr.dual ? 4 : 3) * int64_t(B);
+            max_blocks = (int64_t(pr.maxit) + BB - 1) / BB + 1;
+        };
+        form(coop_g > 0);
+        GraphOwner g;                               // one block of B iterations, captured at its first use
+        auto launch_block = [&] {
+            if (coop && !window(view)) {
+                if (blocks > 0) fail(MSB_ECUDA, "a window of iterations was refused after others had run");
+                form(false);
+            }
+            if (!coop && prof_on()) {
+                for (int i = 0; i < B; ++i) iteration(view);
+            } else if (!coop) {
+                if (!g.exec) {
+                    MSB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+                    for (int i = 0; i < B; ++i) iteration(view);
+                    MSB_CUDA(cudaStreamEndCapture(st, &g.graph));
+                    MSB_CUDA(cudaGraphInstantiate(&g.exec, g.graph, 0));
+                }
+                MSB_CUDA(cudaGraphLaunch(g.exec, st));
+            }
+            launches += per_block;
+        };
         if (prof_on()) {
             // Profiled: direct launches, one sync per block, and one after each fused
             // update to attribute its work (shifts and iterations it carried).
@@ -1372,10 +1417,7 @@ struct SolverImpl {
                 MSB_CUDA(cudaStreamSynchronize(st));
             };
             for (;;) {
-                if (coop) window(view);
-                else
-                    for (int i = 0; i < B; ++i) iteration(view);
-                launches += per_block;
+                launch_block();
                 ++blocks;
                 look();
                 if (coop)
@@ -1395,16 +1437,6 @@ struct SolverImpl {
             prof_collect();
         } else {
 
-        // One block of B iterations, captured once (k_window: launched directly).
-        cudaGraph_t graph = nullptr;
-        cudaGraphExec_t exec = nullptr;
-        if (!coop) {
-            MSB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            for (int i = 0; i < B; ++i) iteration(view);
-            MSB_CUDA(cudaStreamEndCapture(st, &graph));
-            MSB_CUDA(cudaGraphInstantiate(&exec, graph, 0));
-        }
-
         HostBuf<SeedState> hstate(2);
         cudaEvent_t ev[2];
         MSB_CUDA(cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming));
@@ -1413,9 +1445,7 @@ struct SolverImpl {
         // Two blocks in flight: launch block i, then look at the state copied
         // after block i-1.  Blocks launched after convergence return at once.
         while (!finished) {
-            if (coop) window(view);
-            else MSB_CUDA(cudaGraphLaunch(exec, st));
-            launches += per_block;
+            launch_block();
             if ((blocks + 1) * BB % W == 0) { flush(); window_begin(); }
             const int slot = int(blocks & 1);
             MSB_CUDA(cudaMemcpyAsync(&hstate.p[slot], state.p, sizeof(SeedState), cudaMemcpyDeviceToHost, st));
@@ -1432,8 +1462,6 @@ struct SolverImpl {
         MSB_CUDA(cudaStreamSynchronize(st));
         cudaEventDestroy(ev[0]);
         cudaEventDestroy(ev[1]);
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
         }
         out.flushes = blocks * (BB / B);
 
@@ -1500,6 +1528,11 @@ int pick_block(int block, msb_precision prec, int64_t n, int ns) {
 // ----------------------------------------------------------------------------
 // C ABI
 // ----------------------------------------------------------------------------
+// For tests (not part of the header): the calling thread's limits of the solves that follow.
+extern "C" void msb_test_solver_limits(int refuse_cooperative) {
+    msb::g_solver_limits.refuse_cooperative = refuse_cooperative != 0;
+}
+
 static msb_status solve_entry(const char* fname, bool dual, msb_op* A, msb_complex c0, const void* b,
                               const msb_complex* shifts, int n_shifts, double tol, int maxit, int block,
                               msb_precision prec, void* x, int* iters, double* resid, int* converged,

@@ -58,6 +58,12 @@ struct SolveResult {
     msb_status status = MSB_OK;
 };
 
+// Limits of the solves of one thread, lowered by tests to reach the forms that a solve falls back to.
+struct SolverLimits {
+    bool refuse_cooperative = false;      // as if the runtime refused the cooperative launch
+};
+extern thread_local SolverLimits g_solver_limits;
+
 void multishift_solve(msb_op* op, const SolveProblem& pr, SolveResult& out, cudaStream_t st);
 // Lag B of the fused per-shift update: `block` if set, else the autotuned choice
 // for (n, ns, prec) if there is one (autotune.cu), else 4 (FP64) / 8 (FP32).
