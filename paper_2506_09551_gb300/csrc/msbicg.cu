@@ -904,6 +904,8 @@ __global__ void __launch_bounds__(256, 1) k_window(View op, V* ring, int64_t ld,
 // one CTA per SM): the FP32 pipe and DRAM are about balanced at 256 FMAs per 32 bytes of P
 // and x.  48 shifts, n = 2.9 M, per 32 iterations: 3.4 ms as four windows of 8, 2.5 ms with
 // NE = 1 (bound by the coefficient loads), 1.9 ms with NE = 2.
+// Shorter windows (16 or 8 iterations, where the ring of residuals has less memory): NE = 1, two CTAs
+// per SM.  Same update of 1,352 iterations: 80 ms (32), 100 ms (16), 164 ms (8).
 // FP64 (BMAX = 8, NE = 1): bound by the FP64 pipe (8 FMAs per shift, element and
 // iteration); windows with many shifts go to the tensor cores (flush_tc.cuh), and this
 // kernel returns at once.
@@ -1164,8 +1166,8 @@ struct SolverImpl {
     cudaStream_t st;
     int nslot, B, grid_vec, grid_flush, grid_mvm, grid_upd;
     // Window of the per-shift update: 32 iterations in FP32, 56 in FP64 (one contraction on
-    // the tensor cores), whatever the block B of iterations per graph; B when the ring of
-    // residuals would take too much memory.
+    // the tensor cores), whatever the block B of iterations per graph; 32, 16 or B when the ring
+    // of residuals would take too much memory.
     int W = 0, grid_tc = 0;
     bool tc = false;
     TcCoef tcc{};
@@ -1285,9 +1287,17 @@ struct SolverImpl {
                 k_tc_coef<<<(pr.ns + 3) / 4, 128, 0, st>>>(nblk.p, coef64.p, pr.ns, W, nslot, &state.p->slot0,
                                                           &state.p->bnorm, tcc);
             }
-            constexpr int BMAX = std::is_same<V, float2>::value ? 32 : 8, NE = std::is_same<V, float2>::value ? 2 : 1;
-            k_flush<V, BMAX, NE><<<grid_flush, 256, 0, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, pr.rows, pr.rowlen,
-                                                         sh, pr.ns, state.p, W, cnt);
+            auto go = [&](auto kern) {
+                kern<<<grid_flush, 256, 0, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, pr.rows, pr.rowlen, sh, pr.ns,
+                                                 state.p, W, cnt);
+            };
+            if constexpr (std::is_same<V, float2>::value) {
+                if (W == 32) go(k_flush<V, 32, 2>);
+                else if (W == 16) go(k_flush<V, 16, 1>);
+                else go(k_flush<V, 8, 1>);
+            } else {
+                go(k_flush<V, 8, 1>);
+            }
             if constexpr (std::is_same<V, double2>::value) {
                 if (tc)
                     k_flush_tc<<<grid_tc, kTcThreads, kTcSmem, st>>>(ring.p, nslot, ld, Pbuf.p, (V*)pr.x, pr.n_out, pr.rows,
@@ -1317,7 +1327,6 @@ struct SolverImpl {
         B = std::min(pr.block, std::is_same<V, float2>::value ? 16 : 8);
         W = std::is_same<V, float2>::value ? 32 : kTcWindow;
         grid_vec = grid_for(n, 256, 8);
-        grid_flush = std::is_same<V, float2>::value ? grid_for((pr.n_out + 1) / 2, 256, 4) : grid_for(pr.n_out, 256, 8);
         constexpr bool f32 = std::is_same<V, float2>::value;
         rows = op->kind == 2 ? (f32 ? op->plan32 : op->plan64) : row_plan<V>(op, 1);
         if (op->kind == 2) rparts = f32 ? op->parts32.p : op->parts64.p;
@@ -1338,25 +1347,33 @@ struct SolverImpl {
         fz_iter.alloc(ns); fz_coef.alloc(ns);
         resid.alloc(ns);
         shifts_dev.alloc(ns);
-        // The ring comes last, and a long one takes at most 16 GiB and a quarter of the memory
-        // that is left: with less room the window is one block, as small as it can be.
-        const size_t ring_bytes = size_t(W + 1) * ld * sizeof(V);
-        if (ring_bytes > (size_t(16) << 30)) W = B;
-        if (W != B && ring_bytes > (size_t(1) << 30)) {
-            size_t free_b = 0, total_b = 0;
-            MSB_CUDA(cudaMemGetInfo(&free_b, &total_b));
-            if (ring_bytes > free_b / 4) W = B;
-        }
-        try {
-            ring.alloc(size_t(W + 1) * ld);
-        } catch (const Error& e) {
-            if (e.status != MSB_ENOMEM || W == B) throw;
-            cudaGetLastError();
-            W = B;
-            ring.alloc(size_t(W + 1) * ld);
+        // The ring comes last.  A long one takes at most 16 GiB and a quarter of the memory that is
+        // left, so that other threads' solves still find room: with less, the window is shorter,
+        // and one block at the end, as small as it can be.  FP64 windows down to 16 iterations stay
+        // on the tensor cores.
+        const int longest = W;
+        for (const int w : {longest, 32, 16, B}) {
+            if (w > longest || w < B) continue;
+            const size_t bytes = size_t(w + 1) * ld * sizeof(V);
+            if (w > B && bytes > g_solver_limits.ring_bytes) continue;
+            if (w > B && bytes > (size_t(1) << 30)) {
+                size_t free_b = 0, total_b = 0;
+                MSB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+                if (bytes > free_b / 4) continue;
+            }
+            W = w;
+            try {
+                ring.alloc(size_t(w + 1) * ld);
+                break;
+            } catch (const Error& e) {
+                if (e.status != MSB_ENOMEM || w == B) throw;
+                cudaGetLastError();
+            }
         }
         nslot = W + 1;
-        tc = std::is_same<V, double2>::value && W == kTcWindow && ns >= kTcMinShifts;
+        tc = !f32 && W >= 16 && ns >= kTcMinShifts;
+        // two elements per thread for a whole FP32 window only
+        grid_flush = f32 && W == 32 ? grid_for((pr.n_out + 1) / 2, 256, 4) : grid_for(pr.n_out, 256, 8);
         if (tc) {
             tc_list.alloc(ns); tc_cnt.alloc(1); tc_exp.alloc(2 * ns); tc_mul.alloc(2 * ns);
             tc_frag.alloc(size_t((ns + 3) / 4) * kTcSteps * kTcDigits * 32);
@@ -1529,7 +1546,8 @@ int pick_block(int block, msb_precision prec, int64_t n, int ns) {
 // C ABI
 // ----------------------------------------------------------------------------
 // For tests (not part of the header): the calling thread's limits of the solves that follow.
-extern "C" void msb_test_solver_limits(int refuse_cooperative) {
+extern "C" void msb_test_solver_limits(int64_t ring_bytes, int refuse_cooperative) {
+    msb::g_solver_limits.ring_bytes = ring_bytes > 0 ? size_t(ring_bytes) : msb::SolverLimits().ring_bytes;
     msb::g_solver_limits.refuse_cooperative = refuse_cooperative != 0;
 }
 

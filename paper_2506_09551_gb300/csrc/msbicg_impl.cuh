@@ -60,6 +60,7 @@ struct SolveResult {
 
 // Limits of the solves of one thread, lowered by tests to reach the forms that a solve falls back to.
 struct SolverLimits {
+    size_t ring_bytes = size_t(16) << 30; // the ring of seed residuals
     bool refuse_cooperative = false;      // as if the runtime refused the cooperative launch
 };
 extern thread_local SolverLimits g_solver_limits;
