@@ -102,7 +102,7 @@ typedef struct {
     int cf_check;        /* levels between convergence checks (e.g. 50)          */
     int cf_maxdepth;     /* depth cap of the continued fraction                  */
     int seed_index;      /* incident energy used as the seed; -1: nearest to 0   */
-    int block;           /* lag of the fused per-shift update (1..16; 0 = auto)  */
+    int block;           /* iterations per graph of the solve (1..16; 0 = auto)  */
     msb_precision precision;
 } msb_map_params;
 
@@ -406,9 +406,10 @@ msb_status msb_rixs_map(const msb_model *model, const msb_map_params *params,
 /* ------------------------------------------------------------------------ */
 
 /* Timed trials, on the operators of `model`, of the launch choices that leave
- * the results unchanged up to the rounding order of a block reduction: the lag
- * B in {1, 2, 4, 8, 16} of the fused per-shift update of a solve with n_in
- * shifts (FP32 or FP64 per `prec`), and the shape of the row-tiled
+ * the results unchanged up to the rounding order of a block reduction: the
+ * iterations B in {1, 2, 4, 8, 16} per graph of a solve with n_in shifts (FP32 or
+ * FP64 per `prec`; without effect, and left at the default 4 or 8, where a window of
+ * iterations is one cooperative launch), and the shape of the row-tiled
  * continued-fraction apply: threads per CTA (128 or 256) for MSB_FP64; for
  * MSB_FP32_MIXED 1 (one column per CTA, 6 CTAs per SM), 2 (two columns per CTA),
  * 3 (one column, 8 CTAs per SM) or 4 (one column per 512-thread CTA, 4 CTAs per
@@ -416,8 +417,8 @@ msb_status msb_rixs_map(const msb_model *model, const msb_map_params *params,
  * timed with CUDA events as the difference of a 2K- and a K-iteration run (the
  * allocations of a call cancel); an apply shape is taken only if its
  * 32-level continued fraction agrees with the first shape's (relative L2 1e-10
- * in FP64, 1e-4 in FP32), and the fixed default shape is kept unless another is
- * at least 2% faster.  The fastest choices are cached for the whole
+ * in FP64, 1e-4 in FP32), and the fixed default B and shape are kept unless another
+ * is at least 2% faster.  The fastest choices are cached for the whole
  * process, keyed by the problem's shape (intermediate dimension, n_in and
  * precision for B; row length, row count and precision for the threads), and
  * used by every later call that leaves them automatic (params->block or the

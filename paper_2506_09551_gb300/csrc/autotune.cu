@@ -1,14 +1,16 @@
 // Autotuner of the launch choices that leave the results unchanged (up to the
-// rounding of a block reduction): the lag B of the fused per-shift update of the
-// multi-shift solve (1, 2, 4, 8, 16 iterations per flush), and the shape of the
+// rounding of a block reduction): the iterations B per graph of the multi-shift
+// solve (1, 2, 4, 8, 16; convergence is looked at once per graph), and the shape of the
 // row-tiled continued-fraction apply: threads per CTA in FP64 (128 or 256); in FP32
 // one column per CTA at 6 CTAs per SM, two columns per CTA, one column at 8 CTAs
 // per SM, or one column per 512-thread CTA.  Each candidate is
 // timed on the model's own operators with CUDA events, as the difference between
 // a run of 2K and a run of K iterations (or levels), so that the allocations of a
 // call cancel; an apply shape whose fraction disagrees with the first shape's
-// beyond rounding is not taken, and the default shape is kept unless another is
-// at least 2% faster.  The fastest choice is cached per problem shape and used by every
+// beyond rounding is not taken, and the default B or shape is kept unless another is
+// at least 2% faster (the trials of B differ by less than that at L = 14: 1.00 to 1.03 ms
+// per iteration).  Solves whose windows run as one cooperative launch keep the default B,
+// which has no effect there.  The fastest choice is cached per problem shape and used by every
 // call that leaves the choice on automatic (params->block == 0 for B; always for
 // the apply threads).
 #include <chrono>
@@ -107,12 +109,13 @@ static void autotune_impl(const msb_model& m, msb_precision prec, int n_in, Tune
         MSB_CUDA(cudaEventElapsedTime(&ms, e0, e1));
         return double(ms);
     };
-    // 1. lag of the fused per-shift update
+    // 1. iterations per graph
     const int Bs[5] = {1, 2, 4, 8, 16};
     const int K = 32;
     {
         DevBuf<C> X(size_t(n_in) * n_out);
         double best = 1e300;
+        bool cooperative = false;
         for (int i = 0; i < 5; ++i) {
             auto run = [&](int maxit) {
                 SolveProblem pr;
@@ -133,6 +136,7 @@ static void autotune_impl(const msb_model& m, msb_precision prec, int n_in, Tune
                     pr.shifts[k] = make_double2(-4.0 + 16.0 * k / std::max(1, n_in - 1), 0.0);
                 SolveResult sr;
                 multishift_solve(opHp.get(), pr, sr, st);
+                cooperative = sr.cooperative;
             };
             run(K);                                    // warm-up
             const double t1 = timed([&] { run(K); });
@@ -140,6 +144,8 @@ static void autotune_impl(const msb_model& m, msb_precision prec, int n_in, Tune
             out.block_ms[i] = std::max(t2 - t1, 0.0) / K;
             if (out.block_ms[i] < best) { best = out.block_ms[i]; out.block = Bs[i]; }
         }
+        const int d = prec == MSB_FP64 ? 2 : 3;                    // the default, 4 or 8
+        if (cooperative || best > 0.98 * out.block_ms[d]) out.block = Bs[d];
     }
     // 2. the row-tiled continued-fraction apply: threads per CTA (FP64: 128 or 256) or
     // the FP32 shape (1..4)

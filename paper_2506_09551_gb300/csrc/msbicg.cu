@@ -1502,6 +1502,7 @@ struct SolverImpl {
         MSB_CUDA(cudaMemcpyAsync(brk.data(), broken.p, ns * sizeof(int), cudaMemcpyDeviceToHost, st));
         MSB_CUDA(cudaStreamSynchronize(st));
         out.status = msb_status(fs.status);
+        out.cooperative = coop;
         int nconv = 0;
         for (int k = 0; k < ns; ++k) nconv += out.conv[k];
         out.n_converged = nconv;

@@ -56,6 +56,7 @@ struct SolveResult {
     std::vector<int> iters, conv;
     std::vector<double> resid;
     msb_status status = MSB_OK;
+    bool cooperative = false;      // the windows ran as one launch each: `block` had no effect
 };
 
 // Limits of the solves of one thread, lowered by tests to reach the forms that a solve falls back to.
@@ -66,8 +67,8 @@ struct SolverLimits {
 extern thread_local SolverLimits g_solver_limits;
 
 void multishift_solve(msb_op* op, const SolveProblem& pr, SolveResult& out, cudaStream_t st);
-// Lag B of the fused per-shift update: `block` if set, else the autotuned choice
-// for (n, ns, prec) if there is one (autotune.cu), else 4 (FP64) / 8 (FP32).
+// Iterations per graph: `block` if set, else the autotuned choice for (n, ns, prec) if there is
+// one (autotune.cu), else 4 (FP64) / 8 (FP32).
 int pick_block(int block, msb_precision prec, int64_t n = 0, int ns = 0);
 // Autotuned choices (0: none cached).
 int tuned_block(int64_t n, int ns, msb_precision prec);
