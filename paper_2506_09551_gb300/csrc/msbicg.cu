@@ -1188,7 +1188,7 @@ struct SolverImpl {
     DevBuf<double> resid;
     DevBuf<double2> shifts_dev;
     ShiftArrays sh{};
-    int64_t launches = 0;
+    int64_t launches = 0, flushes = 0;
 
     SolverImpl(const SolveProblem& p_, cudaStream_t s) : pr(p_), st(s) {}
 
@@ -1309,6 +1309,7 @@ struct SolverImpl {
                                                                                   pr.rows, pr.rowlen, sh, state.p);
         }
         launches += 1 + (tc ? 2 : 0) + (pr.rrec ? 1 : 0);
+        ++flushes;
     }
 
     void window_begin() {
@@ -1480,7 +1481,7 @@ struct SolverImpl {
         cudaEventDestroy(ev[0]);
         cudaEventDestroy(ev[1]);
         }
-        out.flushes = blocks * (BB / B);
+        out.flushes = flushes;
 
         SeedState fs;
         MSB_CUDA(cudaMemcpyAsync(&fs, state.p, sizeof(SeedState), cudaMemcpyDeviceToHost, st));
