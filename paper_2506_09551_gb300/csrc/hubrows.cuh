@@ -259,15 +259,14 @@ constexpr size_t kMaxRowBytes = 112 * 1024;      // two CTAs per SM
 template <typename V>
 RowPlan row_plan(const msb_op* op, int nvec) {
     RowPlan p;
-    std::vector<const msb_op*> ops;
-    if (op->kind == 0) ops.push_back(op);
-    else if (op->kind == 2) ops = op->parts;
-    else return p;
+    if (op->kind != 0 && op->kind != 2) return p;
+    const msb_op* const* ops = op->kind == 0 ? &op : op->parts.data();      // made for every apply: no heap
+    const size_t nops = op->kind == 0 ? 1 : op->parts.size();
     int64_t maxD = 0;
     constexpr bool f32 = std::is_same<V, float2>::value;
     p.pair = f32;
-    for (const msb_op* o : ops) {
-        const HubView& h = o->hub;
+    for (size_t i = 0; i < nops; ++i) {
+        const HubView& h = ops[i]->hub;
         if (h.hdnr16 == nullptr || h.hup2 != nullptr || h.dirup != nullptr || h.Dup * h.Ddn >= (int64_t(1) << 31)) return p;
         maxD = std::max(maxD, h.Ddn);
         p.pair = p.pair && h.Ddn % 2 == 0;
@@ -275,8 +274,8 @@ RowPlan row_plan(const msb_op* op, int nvec) {
     const int pe = p.pair ? 2 : 1;
     p.threads = maxD >= 1024 * pe ? 256 : 128;
     int64_t t0 = 0;
-    for (size_t i = 0; i < ops.size(); ++i) {
-        HubPart q{};
+    for (size_t i = 0; i < nops; ++i) {
+        HubPart& q = i == 0 ? p.one : p.parts.emplace_back();
         q.v = ops[i]->hub;
         q.off = op->kind == 2 ? op->sum.off[i] : 0;
         q.shift = op->kind == 2 ? op->sum.shift[i] : 0.0;
@@ -285,18 +284,20 @@ RowPlan row_plan(const msb_op* op, int nvec) {
         q.split = 1;
         // halve the rows' work while a column has fewer than ~12 tiles per SM and a part
         // still has two elements per thread
-        while (q.R == 1 && q.split < 4 && q.v.Dup * q.split * int64_t(ops.size()) * nvec < int64_t(sm_count()) * 12 &&
+        while (q.R == 1 && q.split < 4 && q.v.Dup * q.split * int64_t(nops) * nvec < int64_t(sm_count()) * 12 &&
                q.v.Ddn / (2 * q.split) >= 2 * p.threads * pe)
             q.split *= 2;
         const size_t sm = size_t(q.R) * (q.v.Ddn + 2) * sizeof(V) + (3 * (q.v.L + 1) + q.R * q.v.Wup) * sizeof(scalar_t<V>) +
                           size_t(q.R) * (q.v.Wup + 2) * 4;
         p.smem = std::max(p.smem, sm);
         t0 += (q.v.Dup + q.R - 1) / q.R * q.split;
-        p.parts.push_back(q);
+        if (i == 0 && op->kind == 2) {
+            p.parts.reserve(nops);
+            p.parts.push_back(q);
+        }
     }
     p.tiles = t0;
-    p.np = int(ops.size());
-    p.one = p.parts[0];
+    p.np = int(nops);
     const int64_t most = 4096;
     p.grid = int(t0 <= most ? t0 : (t0 + (t0 + most - 1) / most - 1) / ((t0 + most - 1) / most));
     p.ok = p.smem <= kMaxRowBytes && t0 < (int64_t(1) << 31);

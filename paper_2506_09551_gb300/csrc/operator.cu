@@ -239,11 +239,37 @@ struct ApplyEpi {
     __device__ __forceinline__ void finish(double*) const {}
 };
 
+thread_local int g_apply_form = 0;       // tests: 1 rows wherever there is a plan, 2 element by element
+
+// Whether the row-tiled product beats the element-wise one for a plain apply of `work` elements.
+// Staging a row pays by the FP64 pipe and by gathers, and costs a barrier and, with few rows, idle
+// SMs.  Measured, us per call, element by element -> rows (D_up x D_dn elements):
+//   FP64: 13 x 1,716 10 -> 17, 120 x 560 10 -> 15, 15 x 6,435 15 -> 28, 91 x 2,002 22 -> 27,
+//     252 x 252 12 -> 14; 264 x 495 18 -> 18, 286 x 715 26 -> 22, 364 x 1,001 39 -> 34.
+//   FP32, even rows: 66 x 792 10 -> 12, 495 x 792 12.4 -> 14.2; 660 x 462 11.6 -> 10.1,
+//     364 x 2,002 17.6 -> 15.0.
+//   FP32, odd rows (one element per thread): 1,001 x 13 9.8 -> 9.4; 3,003 x 91 10 -> 12,
+//     12,012 x 91 21 -> 28, 924 x 495 12.8 -> 15.6, 420 x 5,005 38 -> 44; 455 x 3,003 32 -> 28,
+//     3,003 x 1,001 61 -> 49.
+template <typename V>
+static bool rows_pay(const RowPlan& p, int64_t work, int nvec) {
+    if (g_apply_form) return g_apply_form == 1;
+    bool single = p.one.R == 1;          // one row per CTA, or a part of it
+    int64_t D = p.one.v.Ddn;
+    for (const HubPart& q : p.parts) {
+        single = single && q.R == 1;
+        D = std::max(D, q.v.Ddn);
+    }
+    if (!std::is_same<V, float2>::value) return !single || 4 * p.tiles * nvec >= 7 * int64_t(sm_count());
+    if (p.pair) return !single || work >= 400000;
+    return work < 200000 ? !single : work >= 1300000 && D >= 256 && D <= 4096;
+}
+
 template <typename V>
 static bool launch_apply_rows(const msb_op* op, double2 c0, const void* x, void* y, int nvec, cudaStream_t st) {
     const bool f32 = std::is_same<V, float2>::value;
     const RowPlan p = op->kind == 2 ? (f32 ? op->plan32 : op->plan64) : row_plan<V>(op, nvec);
-    if (!p.ok) return false;
+    if (!p.ok || !rows_pay<V>(p, op->dim * nvec, nvec)) return false;
     // two adjacent FP32 elements move as 16 bytes: every vector must start on that boundary
     if (p.pair && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u)) return false;
     const int64_t n = op->dim;
@@ -291,6 +317,9 @@ void op_apply(msb_op* op, double2 c0, const void* x, void* y, int nvec, msb_prec
 // ----------------------------------------------------------------------------
 // C ABI: operators
 // ----------------------------------------------------------------------------
+// For tests (not part of the header): the form of the calling thread's applies; 0 chooses by size.
+extern "C" void msb_test_apply_form(int form) { msb::g_apply_form = form; }
+
 extern "C" msb_status msb_op_create_hubbard(const msb_model* model, int intermediate, msb_op** out) {
     return msb::guard("msb_op_create_hubbard", [&] {
         MSB_REQUIRE(model != nullptr && out != nullptr, "NULL argument");

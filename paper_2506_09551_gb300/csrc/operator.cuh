@@ -283,8 +283,8 @@ struct RowPlan {
     int grid = 0;             // CTAs per column (each loops over tiles when tiles > grid)
     size_t smem = 0;
     bool pair = false;        // FP32: every D_dn even, two elements per thread
-    HubPart one{};            // the part of a single operator (passed by value)
-    std::vector<HubPart> parts;
+    HubPart one{};            // the first part; of a single operator the only one (passed by value)
+    std::vector<HubPart> parts;   // all parts of a direct sum
 };
 
 }  // namespace msb
