@@ -21,7 +21,7 @@
 //
 // Measured (GB300, per call, against a thread per element with both species' hops
 // gathered from global memory): eight FP64 vectors on the L = 12 ring (D = 853,776)
-// 1235 -> 514 us (the FP64 pipe alone needs about 410 us); one FP32 vector on the L = 14
+// 1235 -> 535 us (the FP64 pipe alone needs about 410 us); one FP32 vector on the L = 14
 // intermediate sector (D = 10,306,296) 246 -> 130 us; the L = 6 ring (300 states) 15 us
 // either way.
 #pragma once
@@ -238,8 +238,9 @@ __global__ void __launch_bounds__(256) k_hub_rows(HubPart p0, const HubPart* __r
 
 // H x + c0 x from the hop sum and the diagonal.  FP64: `shift` holds the real part of c0 too;
 // it is not folded into the diagonal, whose sum with it would be rounded at the diagonal's
-// size (eight vectors at L = 12: distance from the 64-bit reference 4.3e-17 with the
-// element-wise kernel, 9.6e-17 folded).  FP32: in the order of the element-wise kernels.
+// size (13 hops and the c0 of a solve against exact arithmetic, error in the 2-norm: 7.0e-17 as
+// here, 7.7e-17 element by element, 9.5e-17 folded).  FP32: in the order of the element-wise
+// kernels.
 __device__ __forceinline__ double2 hub_value(double2 acc, double dg, double mt, double shift, double, double c0i, double2 x) {
     return make_double2(fma(mt, acc.x, fma(dg, x.x, fma(shift, x.x, -c0i * x.y))),
                         fma(mt, acc.y, fma(dg, x.y, fma(shift, x.y, c0i * x.x))));

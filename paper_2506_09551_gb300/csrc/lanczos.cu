@@ -1574,11 +1574,11 @@ static void cf_impl(const CFColumns& P, const View& view, const double* w, int n
         if (hn0[c] > 0.0) hcols[nact++] = c;
     cols.upload(hcols.data(), std::max(nact, 1), st);
     const dim3 gridA(unsigned(nblkA), 1);
-    // Two column groups on two streams: the apply of one group (bound by issue and the
-    // L1/shared pipe) overlaps the orth pass of the other (bound by DRAM).  Each group's
-    // levels are ordered on its own stream; the groups meet at every convergence check.
-    // With the profiler on, one group, so that every launch is timed alone.
-    // Small batches gain as well (one group -> two: map of the L = 8 ring, 41 columns of 4,900,
+    // Two column groups on two streams, so that a group's launches fill the SMs that the other's
+    // leave idle at their ends.  Each group's levels are ordered on its own stream; the groups
+    // meet at every convergence check.  With the profiler on, one group, so that every launch is
+    // timed alone.  Where one group's launches fill the chip many times over it gives nothing
+    // (24 columns at L = 12: 46.0 ms with two groups, 45.9 with one); small batches gain (one group -> two: map of the L = 8 ring, 41 columns of 4,900,
     // 70.1 -> 65.7 ms; 60 levels of 16 and 40 columns of 63,504, 4.44 -> 3.89 and 8.70 -> 7.65 ms).
     const int ngrp = prof_on() ? 1 : 2;
     // a column's sums close in its own last CTA where the CTAs per column are few

@@ -567,7 +567,7 @@ __global__ void k_block_begin(SeedState* st, ShiftArrays sh, int ns, int nslot) 
 //
 // With the vectors of an iteration in a few microseconds' reach of the chip, three dependent
 // launches, their fences and the serial scalar work between them decide: 29 us per iteration
-// on the L = 8 ring (n = 3,920), 18 here.  Here the CTAs of one launch keep r, p and v of their elements
+// on the L = 8 ring (n = 3,920), 14.5 here.  The CTAs of one launch keep r, p and v of their elements
 // in registers for the whole window and meet at barriers in global memory (three per
 // iteration): only p (for the gathers of the product, through L2), the residuals for the
 // window's per-shift update and the partial sums leave the SM.  Every worker CTA forms alpha
