@@ -33,7 +33,8 @@
 // faster than the residuals of distant shifts (1e-160 after ~1000 iterations
 // at L = 8), so r_m and zeta^k_m leave the FP32 range long before the shifts
 // converge, and the FP64 range on long runs.  Everything is linear, so the
-// seed vectors r, p, v are stored as S_m times their true values and each
+// seed vectors r, p, v are stored as S_m times their true values (S_0 brings a right-hand side
+// beyond 2^+-300 near one, so that rho, 1 / rho and the squares stay normal numbers) and each
 // shift's (zeta_m, zeta_{m-1}) as g_k times theirs, with S_m and g_k powers of
 // two (exact scaling: no rounding changes).  Only the scalars see the scales:
 //   gamma~ = gamma * S_m / S_{m-1},   c~ = c / S_m = alpha 2^{E_k} / zeta~_{m+1},
@@ -62,7 +63,7 @@ struct SeedState {
     double2 beta;         // beta_m: built p_m (0 at m = 0)
     double2 beta_n, rho_n;   // beta_{m+1}, (r~_{m+1}, r~_{m+1}) before the rescale
     double rn2_n;         // ||r~_{m+1}||^2
-    double2 irho;         // 1 / rho_m (not finite if that is not representable)
+    double2 irho;         // 1 / rho_m
     double2 boa;          // beta_m / alpha_{m-1}
     int f_n, bad_n;       // its rescale exponent; why beta could not be formed
     unsigned cnt_a, cnt_b;   // arrival counters of the two reductions
@@ -72,6 +73,8 @@ struct SeedState {
     double rnorm;         // ||r_m||
     double bnorm;         // ||b||
     double ibnorm;        // 1 / ||b|| (0 for b = 0)
+    double ir0;           // 1 / ||r~_0||
+    int f0;               // log2 S_0: r~_0 = 2^f0 b
     double tol;
     int m;                // iteration count
     int m0;               // iteration at the start of the current block
@@ -123,16 +126,15 @@ __device__ __forceinline__ int form_alpha(double2 mu, double2 rho, double2& a) {
 // beta_{m+1} = rho_{m+1} / rho_m and the exponent f of the rescale, from the sums (rho_{m+1},
 // ||r_{m+1}||^2); why it could not be formed, else MSB_OK.  irho = 1 / rho_m was formed beside the
 // vectors, off the chain (a division here: 2% of the L = 8 solve).
-__device__ __forceinline__ int form_beta(const double (&v)[3], double2 rho, double2 irho, double ibnorm, double2& b, int& f) {
+__device__ __forceinline__ int form_beta(const double (&v)[3], double2 irho, double ir0, double2& b, int& f) {
     b = make_double2(0.0, 0.0);
     f = 0;
     if (!isfinite(v[0]) || !isfinite(v[1]) || !isfinite(v[2])) return MSB_ENONFINITE;
     if (v[2] == 0.0) return MSB_OK;                         // exact solution: every shift converged
     if (v[0] == 0.0 && v[1] == 0.0) return MSB_EBREAKDOWN;  // (r, r) = 0 with r != 0
     b = cmul(make_double2(v[0], v[1]), irho);
-    if (!cfinite(irho)) b = cdiv1(make_double2(v[0], v[1]), rho);       // rho_m is subnormal
-    // bring ||r~|| back near ||b|| once it drifts by more than 2^20
-    const double ratio2 = v[2] * ibnorm * ibnorm;
+    // bring ||r~|| back near ||r~_0|| once it drifts by more than 2^20
+    const double ratio2 = v[2] * ir0 * ir0;
     if (ratio2 < 0x1p-40 || ratio2 > 0x1p40) f = -(ilogb(ratio2) >> 1);
     return MSB_OK;
 }
@@ -427,7 +429,7 @@ __global__ void __launch_bounds__(kVecThreads, 3) k_seed_update(V* ring, int64_t
     if (threadIdx.x == 0) {
         double2 b;
         int f;
-        const int bad = form_beta(acc, st->rho, st->irho, st->ibnorm, b, f);
+        const int bad = form_beta(acc, st->irho, st->ir0, b, f);
         st->beta_n = b;
         st->rho_n = make_double2(acc[0], acc[1]);
         st->rn2_n = acc[2];
@@ -712,7 +714,7 @@ __device__ void window_scalars(SeedState* st, const double* part, int G, const S
                 if (!end) {
                     double2 b;
                     int f;
-                    st->bad_n = form_beta(v, st->rho, st->irho, st->ibnorm, b, f);
+                    st->bad_n = form_beta(v, st->irho, st->ir0, b, f);
                     st->beta_n = b;
                     st->rho_n = make_double2(v[0], v[1]);
                     st->rn2_n = v[2];
@@ -759,7 +761,7 @@ __global__ void __launch_bounds__(256, 1) k_window(View op, V* ring, int64_t ld,
     const int tid = threadIdx.x;
     const int64_t nth = int64_t(G) * blockDim.x, t0 = int64_t(b) * blockDim.x + tid;
     const int slot0 = st->slot0;
-    const double ibnorm = st->ibnorm;
+    const double ir0 = st->ir0;
     double2 rho = st->rho, irho = st->irho;    // used by thread 0 only
     V r[NE], q[NE], v[NE];
 #pragma unroll
@@ -846,7 +848,7 @@ __global__ void __launch_bounds__(256, 1) k_window(View op, V* ring, int64_t ld,
             if (tid == 0) {
                 double2 bt = make_double2(0.0, 0.0);
                 int f = 0, e = bad;
-                if (!e) e = !ok ? int(MSB_ETIMEOUT) : load_l2(&st->stop_at) < j ? int(MSB_EMAXITER) : form_beta(sums, rho, irho, ibnorm, bt, f);
+                if (!e) e = !ok ? int(MSB_ETIMEOUT) : load_l2(&st->stop_at) < j ? int(MSB_EMAXITER) : form_beta(sums, irho, ir0, bt, f);
                 s_c = bt;
                 s_f = f;
                 s_bad = e;
@@ -1090,9 +1092,12 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
     double v[3];
     reduce_partials<3>(part, nblk, v, sm);
     __shared__ double s_bn;
+    __shared__ int s_f0;
     if (threadIdx.x == 0) {
         const double bn = sqrt(v[2]);
-        st->rho = make_double2(v[0], v[1]);
+        const int f0 = bn > 0.0 && isfinite(bn) && !(bn > 0x1p-300 && bn < 0x1p300) ? -ilogb(bn) : 0;
+        st->f0 = f0;
+        st->rho = scale2(make_double2(v[0], v[1]), 2 * f0);
         st->alpha = make_double2(1.0, 0.0);
         st->boa = make_double2(0.0, 0.0);
         st->irho = cdiv1(make_double2(1.0, 0.0), st->rho);
@@ -1100,7 +1105,8 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         st->rnorm = bn;
         st->bnorm = bn;
         st->ibnorm = bn > 0.0 ? 1.0 / bn : 0.0;
-        st->rexp[0] = bn > 0.0 && isfinite(bn) ? ilogb(bn) : 0;
+        st->ir0 = scale2(st->ibnorm, -f0);
+        st->rexp[0] = bn > 0.0 && isfinite(bn) ? ilogb(bn) + f0 : 0;
         st->tol = tol;
         st->m = 0; st->m0 = 0; st->j = 0; st->jcur = 0; st->slot0 = 0;
         st->status = MSB_OK;
@@ -1114,11 +1120,12 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         st->bar_a = 0;
         st->stop_at = INT_MAX;
         st->stop = (bn == 0.0 || maxit <= 0) ? 1 : 0;
-        if (bn != 0.0 && st->rho.x == 0.0 && st->rho.y == 0.0) { st->status = MSB_EBREAKDOWN; st->stop = 1; }
+        if (bn != 0.0 && v[0] == 0.0 && v[1] == 0.0) { st->status = MSB_EBREAKDOWN; st->stop = 1; }
         st->nactive = bn == 0.0 ? 0 : ns;
         st->fexp = 0;
-        st->sexp = 0;
+        st->sexp = f0;
         s_bn = bn;
+        s_f0 = f0;
     }
     __syncthreads();
     for (int k = threadIdx.x; k < ns; k += blockDim.x) {
@@ -1132,9 +1139,24 @@ __global__ void __launch_bounds__(kScalarThreads) k_init_state(SeedState* st, co
         sh.nblk[k] = 0;
         sh.iters[k] = 0;
         sh.resid[k] = 0.0;
-        sh.zexp[k] = 0;
+        sh.zexp[k] = -s_f0;
         sh.fz_coef[k] = make_double2(1.0, 0.0);
         sh.fz_iter[k] = 0;
+    }
+}
+
+// r~_0 = p_0 = 2^f0 b (dual form: the dual vectors too).
+template <typename V>
+__global__ void __launch_bounds__(256) k_init_scale(V* ring, V* p, int64_t n, const SeedState* __restrict__ st, V* rt, V* pt) {
+    if (st->f0 == 0) return;
+    const double sc = scale2(1.0, st->f0);
+    for (int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; s < n; s += int64_t(gridDim.x) * blockDim.x) {
+        ring[s] = cscale(sc, 0.0, ring[s]);
+        p[s] = cscale(sc, 0.0, p[s]);
+        if (rt) {
+            rt[s] = cscale(sc, 0.0, rt[s]);
+            pt[s] = cscale(sc, 0.0, pt[s]);
+        }
     }
 }
 
@@ -1395,7 +1417,11 @@ struct SolverImpl {
             k_init_state<<<1, kScalarThreads, 0, st>>>(state.p, part.p, grid_vec, sh, shifts_dev.p, int(ns),
                                                         pr.tol, pr.maxit);
         }
-        launches += 2;
+        {
+            ProfScope ps("shift_scalars", st, 0, 0);
+            k_init_scale<V><<<grid_vec, 256, 0, st>>>(ring.p, p.p, n, state.p, rt.p, pt.p);
+        }
+        launches += 3;
         MSB_LAUNCH_CHECK();
         bool coop = false;
         int BB = 0;                                 // iterations per launch of a block
