@@ -298,7 +298,7 @@ msb_status msb_ground_state_noalloc(msb_op *H, double tol, int maxit, const doub
  * looked at.  The vectors p^(k), x^(k) are advanced once per window of 56 (FP64) or 32
  * (FP32) iterations from the stored seed residuals, with coefficients from the same
  * recurrences; the window is 32, 16 or `block` when the residuals would take more than 16 GiB
- * or a quarter of the free memory.
+ * or a quarter of the free memory, or maxit is at most half the window.
  * Returns MSB_EMAXITER (results still written) if a shift did not converge
  * within maxit, MSB_EBREAKDOWN / MSB_ENONFINITE on a failed recurrence,
  * MSB_EINVAL for an operator with Peierls phases (not complex symmetric: use

@@ -116,3 +116,16 @@ def test_breakdown_in_a_later_window(limits, block):
     shifts = np.array([0.0, 0.25 + 0.5j, 0.375 + 0.5j])
     x, per, seeds, info, st = op.multishift_reseeded(b, shifts, maxit=100, max_seeds=1, block=block)
     assert info["iterations"] == 2 and np.all(per["dr"] <= 32 * 2.0 ** -53 * 3.0 ** 0.5), per["dr"]
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_capped_solves_take_no_longer_ring(cuda, prec):
+    """Workspace of a solve of a few iterations: no more residuals than it can have."""
+    from paper_2506_09551_gb300 import api
+    op = _operator("ring")
+    b = torch.tensor(workloads.random_complex_rhs(op.dim, 5), dtype=api.cdtype(prec), device="cuda")
+    size = [op.multishift_solve(b, [0.0], C0, tol=0.0, maxit=m, block=4, prec=prec, allow_status=(5,))[2]["device_bytes"]
+            for m in (3, 8, 9, 16, 17, 100)]
+    slot = op.dim * (8 if prec else 16)
+    assert size[1] - size[0] == 0 and size[2] - size[1] == 12 * slot and size[3] == size[2]
+    assert size[4] - size[3] == 16 * slot and size[5] - size[4] == (0 if prec else 24 * slot)
